@@ -398,7 +398,7 @@ __global__ void __launch_bounds__(kConvThreads, 1)
     }
   } else if (warp == kWarpMma || warp == kWarpMma2) {
     // =================== MMA issue ===================
-    // Two MMA warps take alternate pairs of K stages of every tile into the same accumulator:
+    // Two MMA warps take alternate pairs of K stages into the same accumulator:
     // one thread issuing tcgen05.mma costs more per instruction than an N <= 128 MMA takes on
     // the tensor pipe.  Every MMA accumulates into a buffer that
     // the epilogue left zeroed, so the order of the two warps' MMAs does not matter (the fp32
@@ -406,7 +406,10 @@ __global__ void __launch_bounds__(kConvThreads, 1)
     // lane issues and commits.
     const int mi = warp == kWarpMma2 ? 1 : 0;
     constexpr uint32_t idesc = idesc_e4m3_f32(kBM, BN);
-    int gp = 0;   // pairs of K stages seen so far (pairs alternate between the two warps)
+    // A pair is two ring slots (2i, 2i + 1), so a slot always belongs to the same warp, which takes its uses
+    // in order: the parity waits are then unambiguous.  (Pairs counted from each tile's first stage moved
+    // over the slots where a tile has an odd number of stages, and a warp could then pass a wait for a
+    // slot whose stage before that, the other warp's, a slower gather group had not filled yet.)
     bool ok = true;
 #pragma unroll 1
     for (int jt = 0; jt < n_local && ok; ++jt) {
@@ -416,11 +419,13 @@ __global__ void __launch_bounds__(kConvThreads, 1)
       tc_fence_after();
       const uint32_t dacc = tmem + (uint32_t)(ab * BN);
       // stages k, k+1 of this tile (one vote, fence and elect for up to 8 MMAs)
+      int step = 1;
 #pragma unroll 1
-      for (int k = 0; k < nk; k += 2, ++gp) {
-        if ((gp & 1) != mi) continue;
-        const bool two = k + 1 < nk;
+      for (int k = 0; k < nk; k += step) {
         const int it = jt * nk + k;   // position in the CTA's stage sequence
+        const bool two = (it & 1) == 0 && k + 1 < nk;
+        step = two ? 2 : 1;
+        if (((it >> 1) & 1) != mi) continue;
         const int s0 = it % kS, s1 = (it + 1) % kS;
         const uint32_t ph0 = (uint32_t)(it / kS) & 1u, ph1 = (uint32_t)((it + 1) / kS) & 1u;
         bool got = mbar_wait(full(s0), ph0);
