@@ -99,6 +99,9 @@ int ifq_version(void);
  *   IFQ_WIN          = 0: never take the window path (IFQ_PATH_WIN requests take the tensor-core path).
  *   IFQ_WARP         = 0: never take the warp-MMA path (IFQ_PATH_WARP requests take the tensor-core
  *                      path).
+ *   IFQ_BAND         = 0: the tensor-core path always runs its im2col kernel; 2 .. 7: its band kernel in
+ *                      that launch shape where the layer and the shape fit (by default the faster of
+ *                      the two, estimated).  The next three ask for the im2col kernel.
  *   IFQ_TC_BN        = 32 / 64 / 128: the tensor-core kernel's output-channel tile width.
  *   IFQ_TC_KS        = 1 / 2: forbid / force splitting K over clusters of two CTAs (by default only
  *                      layers that would leave more than half of the SMs idle are split).

@@ -7,6 +7,7 @@
 #include <cudaTypedefs.h>
 
 #include <cstdint>
+#include <cmath>
 #include <cstdlib>
 #include <cstring>
 #include <mutex>
@@ -14,6 +15,7 @@
 #include <utility>
 #include <vector>
 
+#include "conv_band.cuh"
 #include "conv_bitserial.cuh"
 #include "conv_direct.cuh"
 #include "conv_tc.cuh"
@@ -216,6 +218,8 @@ cudaError_t set_warp_attrs() {
   return e;
 }
 
+cudaError_t set_band_attrs();
+
 // Per-device one-time setup (shared-memory limits of the kernels, SM count).
 int ensure_init(int* nsm_out, bool* stack_ok = nullptr) {
   int dev = 0;
@@ -236,7 +240,7 @@ int ensure_init(int* nsm_out, bool* stack_ok = nullptr) {
         cudaFuncSetAttribute(conv_win_kernel<1, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, kWinMaxSmem) !=
             cudaSuccess)
       return IFQ_ECUDA;
-    if (set_warp_attrs() != cudaSuccess) return IFQ_ECUDA;
+    if (set_warp_attrs() != cudaSuccess || set_band_attrs() != cudaSuccess) return IFQ_ECUDA;
     if (cudaDeviceGetAttribute(&d.nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return IFQ_ECUDA;
     if (cudaFuncSetAttribute(conv_stack_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, StackSmem::bytes) !=
         cudaSuccess)
@@ -344,8 +348,42 @@ size_t prep_masks_offset(const ifq_conv_desc* d, const ConvGeom& g) {
 // 8-bit-input layers keep their masks.
 size_t prep_pbits_offset(const ifq_conv_desc* d, const ConvGeom& g) { return prep_masks_offset(d, g); }
 
+// Geometry of the band path (conv_band.cuh) that depends on the layer alone, or false where the path does
+// not apply.  It takes 2-, 3- or 4-bit codes without a fused pool, stride 1 or a 1 x 1 filter, at most
+// kBandMaxTaps filter taps, more than 32 output channels and an accumulator magnitude inside the checked exact
+// range.  Filters that cover their whole unpadded input (fully connected layers) are left out: a 6 x 6 x 256 ->
+// 4096 layer at batch 128 measured 30.5 us here (as a 1 x 1 layer on the flattened input) against 13.7 us on
+// the im2col kernel, which splits K.
+struct BandGeom {
+  int fields, dig;                            // 2-bit fields per pixel, digits per code
+  int taps, planes, npair, nodd, cols, crows;
+};
+
+bool band_geom(const ifq_conv_desc* d, const ConvGeom& g, BandGeom* b) {
+  if (g.in8 || g.pool != 1 || d->cout <= 32 || (long long)g.lvl * g.K > kTcMaxAcc) return false;
+  b->taps = d->kh * d->kw;
+  if (b->taps > kBandMaxTaps || (d->stride != 1 && b->taps != 1)) return false;
+  if (b->taps > 1 && d->pad == 0 && d->kh == d->h && d->kw == d->w) return false;
+  b->dig = g.sb / 2;
+  b->fields = d->cin * b->dig;
+  b->planes = ceil_div(b->fields, 32);
+  b->npair = b->planes / 2;
+  b->nodd = b->planes % 2 ? band_odd_steps(b->taps) : 0;
+  b->cols = 2 * (b->npair * b->taps + b->nodd);
+  b->crows = (int)round_up((size_t)d->cout, (size_t)kBandBlock);
+  return true;
+}
+
+// Layers on codes: then the band path's filters, [core column][cout][16 bytes].
+size_t prep_band_offset(const ifq_conv_desc* d, const ConvGeom& g) {
+  return round_up(prep_pbits_offset(d, g) + (size_t)d->cout * g.Kpad / 8, 256);
+}
+
 size_t prep_bytes(const ifq_conv_desc* d, const ConvGeom& g) {
-  return g.in8 ? prep_masks_offset(d, g) + (size_t)g.K * 4 : prep_pbits_offset(d, g) + (size_t)d->cout * g.Kpad / 8;
+  if (g.in8) return prep_masks_offset(d, g) + (size_t)g.K * 4;
+  BandGeom b;
+  if (!band_geom(d, g, &b)) return prep_pbits_offset(d, g) + (size_t)d->cout * g.Kpad / 8;
+  return prep_band_offset(d, g) + (size_t)b.cols * b.crows * 16;
 }
 
 bool tc_supported(const ifq_conv_desc* d, const ConvGeom& g);
@@ -611,8 +649,7 @@ int choose_path(const ifq_conv_desc* d, const ConvGeom& g) {
 // 52 / 54 / 72 at BN = 32 / 64 / 128, independent of whether consecutive MMAs
 // share an accumulator), a K stage issues 4 of them, and the makespan is
 // ceil(tiles / SMs) * nk * 4 * t(BN).  Ties go to the wider tile.
-int choose_bn(const ConvGeom& g, int cout, int nsm) {
-  const int forced = env_int("IFQ_TC_BN", 0);
+int choose_bn(const ConvGeom& g, int cout, int nsm, int forced) {
   if (forced == 32 || forced == 64 || forced == 128) return forced;
   int best = 32;
   double best_cost = 1e300;
@@ -648,10 +685,9 @@ int tc_max_clusters(int bn, int ks, int nsm) {
 // layer would leave more than half of the SMs idle, the split grid fits in one wave of clusters and
 // every CTA keeps at least eight K stages.  IFQ_TC_KS = 1 / 2 forbids / forces it where eligible.
 template <int GB, int SB, int SBO>
-void choose_split(const ConvGeom& g, int cout, int nsm, int* bn, int* ks) {
+void choose_split(const ConvGeom& g, int cout, int nsm, int forced, int* bn, int* ks) {
   *ks = 1;
   if constexpr (GB == 16) {
-    const int forced = env_int("IFQ_TC_KS", 0);
     if (forced == 1) return;
     const int nk = g.Kpad / kBK;
     if (cout <= 32 || nk < 4) return;   // the split instance is BN = 64, KS = 2
@@ -757,6 +793,213 @@ void fill_conv_args(const ifq_conv_desc* d, const ConvGeom& g, int bn, const voi
   a->div_pwo = make_fastdiv((uint32_t)g.pwo);
 }
 
+// ---------------------------------------------------------------- band path
+
+// Slots between rows (or rows between images): the smallest pitch for which what a row needs past it is
+// zero padding on both sides, so the end of a row and the start of the next share their slots.
+int band_pitch(int out, int in, int k, int s, int pad) {
+  const int need = out + k - 1;
+  for (int P = out; P < need; ++P)   // slots P .. need - 1 are right padding of a row and left padding of the next
+    if (need - P <= P && s * P - pad >= in && s * (need - 1 - P) < pad) return P;
+  return need;
+}
+
+// TMA descriptor of the band path's filters as rows of 8-byte elements, one row per core column: boxes of bn
+// filter rows x 8 core columns (one filter stage), no swizzle.
+bool encode_bandmap(const ifq_conv_desc* d, const ConvGeom& g, const void* w_prep, int bn, CUtensorMap* tm) {
+  BandGeom b;
+  if (!get_encode() || !band_geom(d, g, &b)) return false;
+  cuuint64_t gdim[2] = {(cuuint64_t)b.crows * 2, (cuuint64_t)b.cols};
+  cuuint64_t gstride[1] = {(cuuint64_t)b.crows * 16};
+  cuuint32_t box[2] = {(cuuint32_t)bn * 2, 8};
+  cuuint32_t estr[2] = {1, 1};
+  return g_encode(tm, CU_TENSOR_MAP_DATA_TYPE_UINT64, 2, (uint8_t*)const_cast<void*>(w_prep) + prep_band_offset(d, g),
+                  gdim, gstride, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
+                  CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+constexpr int kBandMaxStages = 64, kBandMaxRing = 16;
+
+// Launch shapes of the band kernel: channel tile, 128-anchor subtiles per tile, channel tiles per CTA, and
+// whether the filters stay in shared memory (with one subtile they do).
+struct BandShape {
+  int bn, mt, ngrp;
+  bool resident;
+};
+// Of 48 shapes timed on 78 layers (the benchmark networks' and random ones) these are within 2 % of the best of
+// all on average; more channel tiles per CTA, streamed filters with one subtile, tiles of 32 channels and two
+// CTAs per SM gained little anywhere.
+constexpr BandShape kBandShapes[] = {{64, 1, 1, true},  {64, 1, 2, true},  {64, 2, 1, true},
+                                     {128, 1, 1, true}, {128, 1, 2, true}, {128, 2, 1, false}};
+constexpr int kBandShapeCount = (int)(sizeof(kBandShapes) / sizeof(kBandShapes[0]));
+constexpr size_t kBandSmem = 232448;
+
+struct BandPlan {
+  BandArgs a;
+  int bn, grid;
+  size_t smem;
+  double cost;             // estimated cycles
+};
+
+// Fills the part of the plan that no launch shape changes.
+void band_fill(const ifq_conv_desc* d, const ConvGeom& g, const BandGeom& b, BandArgs* a) {
+  memset(a, 0, sizeof(*a));
+  a->n = d->n; a->h = d->h; a->w = d->w; a->pb = b.fields / 4;
+  a->cout = d->cout; a->lvl = g.lvl; a->bound = g.lvl * g.K;
+  a->oh = g.ho; a->ow = g.wo;
+  a->pad = d->pad; a->kh = d->kh; a->kw = d->kw; a->s = d->stride;
+  a->P = band_pitch(a->ow, a->w, a->kw, a->s, a->pad);
+  a->HP = band_pitch(a->oh, a->h, a->kh, a->s, a->pad);
+  a->linear = a->s == 1 && a->pad == 0 && a->P == a->w && a->HP == a->h ? 1 : 0;
+  a->planes = b.planes; a->taps = b.taps; a->nodd = b.nodd;
+  a->nstep = b.cols / 2;
+  a->gran = a->pb % 16 == 0 ? 16 : (a->pb % 8 == 0 ? 8 : (a->pb % 4 == 0 ? 4 : (a->pb % 2 == 0 ? 2 : 1)));
+  a->div_P = make_fastdiv((uint32_t)a->P);
+  a->div_HP = make_fastdiv((uint32_t)a->HP);
+}
+
+// One launch shape on `base` (band_fill): fills the plan, or false where it does not fit.
+bool band_try(const BandArgs& base, const BandShape& sh, int sbo, int nsm, BandPlan* pl) {
+  pl->a = base;
+  BandArgs& a = pl->a;
+  const int bn = sh.bn, mt = sh.mt;
+  const long long anchors = (long long)a.n * a.HP * a.P;
+  a.mt = mt;
+  const int maxoff = (a.kh - 1) * a.P + a.kw - 1;
+  a.slots = (int)round_up((size_t)(128 * mt + maxoff + 1), 8);
+  // 32-bit slot and input-pixel indexes (a warp may look up to one batch past the last slot)
+  if (anchors + a.slots + 4096 >= (1LL << 31) || (long long)a.n * a.h * a.w >= (1LL << 31)) return false;
+  if (a.nodd && a.P < a.kw) return false;   // the second tap of a pair lies behind the first
+  a.mtiles = (int)((anchors + 128 * mt - 1) / (128 * mt));
+  a.plane_bytes = (uint32_t)a.slots * 16u;
+  a.nt = ceil_div(a.cout, bn);
+  a.ngrp = sh.ngrp;
+  if (a.ngrp > a.nt) return false;
+  a.ngroups = ceil_div(a.nt, a.ngrp);
+  if (a.ngroups > nsm) return false;
+  const int kacc = (kBandCols - 16) / bn;
+  a.nacc = mt == 2 ? kacc & ~1 : kacc;          // (even: see band_mma)
+  a.ncb = a.nacc & 1 ? 2 * a.nacc : a.nacc;
+  // shared memory: the band ring, filters, then lines and tables
+  a.stage_bytes = (uint32_t)(4 * 2 * bn * 16);
+  a.resident = sh.resident ? 1 : 0;
+  const size_t cols = (size_t)a.ngrp * bn, thrb = sbo == 2 ? 16 : 80;
+  // Planes per chunk: as many as a granule's lanes take at once and leave a ring of two (deeper rings and
+  // smaller chunks measured no faster: 178 to 183 us on the 3x3 256 -> 256 layer, 50 to 53 us on the 1x1
+  // 512 -> 512 one with whole 8-plane chunks against 71 us with 4).
+  const int cpmax = a.gran == 16 ? 8 : 4;
+  size_t bbytes = 0;
+  for (int cp = std::min(a.planes, cpmax); cp >= 1 && a.ring == 0; cp = cp > 2 ? (cp - 1) / 2 * 2 : 0) {
+    if (cp < a.planes && (cp & 1)) continue;
+    const int nchunk = ceil_div(a.planes, cp), pl_last = a.planes - (nchunk - 1) * cp;
+    const int s_full = cp / 2 * a.taps, s_last = pl_last / 2 * a.taps + (pl_last & 1 ? a.nodd : 0);
+    const int nst = (nchunk - 1) * ceil_div(s_full, 4) + ceil_div(s_last, 4);
+    const long long all = (long long)a.ngrp * nst;
+    if (a.resident && all > kBandMaxStages) continue;
+    const int stages = a.resident ? (int)all : 8;
+    const int tab_last = nchunk > 1 ? (int)round_up((size_t)s_full, 4) : 0;
+    const int ntab = tab_last + (int)round_up((size_t)s_last, 4);
+    const size_t cb = (size_t)cp * a.plane_bytes;
+    const size_t rest = (size_t)stages * a.stage_bytes + cols * (8 + thrb) + 256 + (size_t)ntab * 4 + 16 +
+                        8 * (size_t)(2 * kBandMaxRing + 2 * stages + 4 * kacc + 3) + 4 * 128;
+    if (rest > kBandSmem) continue;
+    const int ring = (int)std::min((kBandSmem - rest) / cb, (size_t)std::min(kBandMaxRing, std::max(3, 2 * nchunk)));
+    if (ring < 2 || (a.ngrp > 1 && ring < nchunk + 1)) continue;
+    a.cp = cp; a.nchunk = nchunk; a.ring = ring;
+    a.stages = stages; a.nst = nst;
+    a.tab_last = tab_last; a.ntab = ntab;
+    a.chunk_bytes = (uint32_t)cb;
+    bbytes = (size_t)stages * a.stage_bytes;
+  }
+  if (a.ring == 0) return false;
+  const int ng = a.gran == 16 ? ceil_div(a.cp, 2) : a.cp;
+  a.glg = ng >= 3 ? 2 : (ng == 2 ? 1 : 0);
+  a.off_b = (uint32_t)round_up((size_t)a.ring * a.chunk_bytes, 128);
+  a.off_lin = a.off_b + (uint32_t)bbytes;
+  a.off_thr = a.off_lin + (uint32_t)cols * 8;
+  a.off_bad = a.off_thr + (uint32_t)(cols * thrb);
+  a.off_tab = a.off_bad + 256;
+  a.off_bar = (uint32_t)round_up((size_t)a.off_tab + (size_t)a.ntab * 4 + 16, 16);   // (a group of entries is read ahead)
+  pl->smem = 128 + a.off_bar + 8 * (size_t)(2 * a.ring + 2 * a.stages + 4 * kacc + 3);
+  if (pl->smem > kBandSmem) return false;
+  const int per = std::max(1, std::min(a.mtiles, nsm / a.ngroups));
+  pl->grid = per * a.ngroups;
+  pl->bn = bn;
+  // Estimated cycles, with constants fitted to 62 layers timed in each shape (10 % from the measured time on
+  // average; the shape picked is within 0.6 % of the best one on average).  What each role of a CTA takes for
+  // one tile; the slowest of them sets the pace after the first tile.
+  const bool wide = sbo == 4, acc = a.y_acc != nullptr;
+  const double units = (double)a.ngrp * mt;
+  const double mma = a.nstep * units * (bn == 128 ? 93.3 : 72.4) * (mt == 2 ? 0.938 : 0.854) + 559.0 * a.ngrp;
+  const double epi = (bn == 128 ? 2140.0 : 1180.0) * (acc ? 4.5 : 1.0) * (wide ? 1.26 : 1.0);
+  const double batches = std::ceil((double)a.slots * (1 << a.glg) / (32.0 * 4 * kBandProd));
+  const double chunk = batches * 1380.0 * (a.gran < 8 ? 2.14 : 1.0) + 297.0;
+  const double fbytes = (double)a.nst * a.ngrp * a.stage_bytes;
+  const double stream = a.resident ? 0.0 : fbytes * 0.0355, fill = a.resident ? fbytes * 0.0174 : 0.0;
+  const double pace = std::max(std::max(mma, units * epi / 2), std::max(a.nchunk * chunk, stream));
+  const double tiles = ceil_div(a.mtiles, per);
+  pl->cost = 4800.0 + (wide ? 2460.0 : 0.0) + std::max(fill, chunk) + 0.7 * mma + epi + (tiles - 0.7) * pace;
+  return true;
+}
+
+// The launch shape of the band path with the smallest estimated time, or false where none fits or the im2col
+// kernel (tc_cost, in cycles) is as fast.  IFQ_BAND: 0: none; 2, 3, ..: that shape of the table, where it fits.
+bool band_plan(const ifq_conv_desc* d, const ConvGeom& g, int nsm, bool acc, double tc_cost, BandPlan* best) {
+  BandGeom b;
+  if (!band_geom(d, g, &b)) return false;
+  const int want = env_int("IFQ_BAND", 1);
+  if (want == 0) return false;
+  if (want == 1 && 0.95 * tc_cost < 8500.0) return false;   // no estimate of band_try is below
+  BandArgs base;
+  band_fill(d, g, b, &base);
+  base.y_acc = acc ? (int32_t*)16 : nullptr;
+  bool have = false;
+  for (int i = 0; i < kBandShapeCount; ++i) {
+    BandPlan p;
+    if (want >= 2 ? want - 2 != i : kBandShapes[i].bn == 128 && d->cout <= 64) continue;
+    if (band_try(base, kBandShapes[i], g.sb, nsm, &p) && (!have || p.cost < best->cost)) {
+      *best = p;
+      have = true;
+    }
+  }
+  return have && (want >= 2 || best->cost < 0.95 * tc_cost);
+}
+
+template <int BN, int SBO>
+struct BandInst {
+  static constexpr auto kern = conv_band_kernel<BN, SBO>;
+  static cudaError_t set_attr() {
+    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBandSmem);
+  }
+  static cudaError_t launch(const BandPlan& p, const CUtensorMap& tm, cudaStream_t st) {
+    return launch_k(kern, dim3((unsigned)p.grid), dim3(kBandThreads), p.smem, st, tm, p.a);
+  }
+};
+
+// f(instance) for the instance of a plan.
+template <typename F>
+cudaError_t band_dispatch(int bn, int sbo, F&& f) {
+  if (bn == 64) return sbo == 2 ? f(BandInst<64, 2>{}) : f(BandInst<64, 4>{});
+  return sbo == 2 ? f(BandInst<128, 2>{}) : f(BandInst<128, 4>{});
+}
+
+cudaError_t set_band_attrs() {
+  cudaError_t e = cudaSuccess;
+  for (int c = 0; c < 4 && e == cudaSuccess; ++c)
+    e = band_dispatch(c & 1 ? 64 : 128, c & 2 ? 2 : 4, [](auto inst) { return decltype(inst)::set_attr(); });
+  return e;
+}
+
+// Estimated cycles of the im2col kernel (conv_tc.cuh) on a layer of codes with tiles of bn channels, K split over
+// ks CTAs: constants fitted as the band kernel's.
+double tc_cycles(const ConvGeom& g, int cout, int nsm, int bn, int ks, int gb, bool acc) {
+  const double tiles = (double)ceil_div(g.M, kBM) * ceil_div(cout, bn), rounds = std::ceil(tiles / nsm);
+  const double stage = (gb == 16 ? 382.0 : (gb == 8 ? 394.0 : (gb == 4 ? 747.0 : 1900.0))) * (g.sb == 4 ? 1.51 : 1.0);
+  const double k = (double)(g.Kpad / kBK) / ks * stage;
+  const double e = (bn == 32 ? 2450.0 : (bn == 64 ? 2430.0 : 4110.0)) * (g.sb == 4 ? 1.5 : 1.0) * (acc ? 2.02 : 1.0);
+  return 5050.0 + (ks == 2 ? 3950.0 : 0.0) + k + e + (rounds - 1) * std::max(k, e);
+}
+
 // early: the kernels before this one in the stream write neither w_prep nor thr / sign (a layer of a
 // stack after the first), so the tensor-core kernel may load them before its dependency wait.
 int run_conv(const ifq_conv_desc* d, const void* x, const void* w_prep, const int32_t* thr, const int8_t* sign,
@@ -840,41 +1083,56 @@ int run_conv(const ifq_conv_desc* d, const void* x, const void* w_prep, const in
     else if (ya) e = launch_k(conv_win_kernel<0, 1>, grid, block, smem, st, tma, wa);
     else e = launch_k(conv_win_kernel<0, 0>, grid, block, smem, st, tma, wa);
   } else if (path == IFQ_PATH_TC) {
-    int bn = choose_bn(g, d->cout, nsm), ks = 1;
+    // (a switch of the im2col kernel's asks for that kernel)
+    const int bn_env = env_int("IFQ_TC_BN", 0), ks_env = env_int("IFQ_TC_KS", 0), bx_env = env_int("IFQ_TC_BX", 0);
+    int bn = choose_bn(g, d->cout, nsm, bn_env), ks = 1;
     const int gb = granule_bytes(d, g);
     if (gb == 16) {
-      if (g.sbi == 2) choose_split<16, 2, 2>(g, d->cout, nsm, &bn, &ks);
-      else if (g.sb == 4) choose_split<16, 4, 4>(g, d->cout, nsm, &bn, &ks);
-      else choose_split<16, 4, 2>(g, d->cout, nsm, &bn, &ks);
+      if (g.sbi == 2) choose_split<16, 2, 2>(g, d->cout, nsm, ks_env, &bn, &ks);
+      else if (g.sb == 4) choose_split<16, 4, 4>(g, d->cout, nsm, ks_env, &bn, &ks);
+      else choose_split<16, 4, 2>(g, d->cout, nsm, ks_env, &bn, &ks);
     }
-    ConvArgs a;
-    fill_conv_args(d, g, bn, x, thr, sign, yc, ya, &a);
-    a.early = early ? 1 : 0;
-    a.wbits = g.in8 ? nullptr : (const uint8_t*)w_prep + prep_pbits_offset(d, g);
-    // Filter tiles expanded from sign bits in shared memory (the split instance only, its TMA warp
-    // streaming the bits): opt-in.  It reads 1 bit per weight from DRAM instead of an e4m3 byte, but
-    // on AlexNet's FC layers (b128) it measured 22.4 / 16.3 us against 20.6 / 16.4 us for FC6 / FC7:
-    // those single-tile launches are bound by the K-stage pipeline's latency, not by the filter
-    // stream.  IFQ_TC_BX = 1 takes it where the filters are read about once (at most two 128-row
-    // tiles), 2 wherever the split instance runs.
-    const int bx_env = env_int("IFQ_TC_BX", 0);
-    const bool bx = bx_env != 0 && (bx_env == 2 || ceil_div(g.M, kBM) <= 2) && bn == 64 && ks == 2 && gb == 16 &&
-                    g.sbi == 2 && g.sb == 2;
-    CUtensorMap tm;
-    if (!(bx ? encode_bitmap(d, g, w_prep, bn, &tm) : encode_wmap(d, g, w_prep, bn, &tm))) return IFQ_ECUDA;
-    if (g.sbi == 2 && g.sb == 2) {
-      if (gb == 16) e = launch_tc_gb<16, 2, 2>(bn, ks, tm, a, nsm, st, bx);
-      else if (gb == 8) e = launch_tc_gb<8, 2, 2>(bn, ks, tm, a, nsm, st);
-      else if (gb == 4) e = launch_tc_gb<4, 2, 2>(bn, ks, tm, a, nsm, st);
-      else e = launch_tc_gb<1, 2, 2>(bn, ks, tm, a, nsm, st);
-    } else if (g.sb == 4) {
-      if (gb == 16) e = launch_tc_gb<16, 4, 4>(bn, ks, tm, a, nsm, st);
-      else if (gb == 8) e = launch_tc_gb<8, 4, 4>(bn, ks, tm, a, nsm, st);
-      else e = launch_tc_gb<4, 4, 4>(bn, ks, tm, a, nsm, st);
-    } else {   // 8-bit input values, 2-bit output codes
-      if (gb == 16) e = launch_tc_gb<16, 4, 2>(bn, ks, tm, a, nsm, st);
-      else if (gb == 8) e = launch_tc_gb<8, 4, 2>(bn, ks, tm, a, nsm, st);
-      else e = launch_tc_gb<4, 4, 2>(bn, ks, tm, a, nsm, st);
+    BandPlan bp;
+    if (!bn_env && !ks_env && !bx_env &&
+        band_plan(d, g, nsm, ya != nullptr, tc_cycles(g, d->cout, nsm, bn, ks, gb, ya != nullptr), &bp)) {
+      CUtensorMap tm;
+      if (!encode_bandmap(d, g, w_prep, bp.bn, &tm)) return IFQ_ECUDA;
+      bp.a.x = (const uint8_t*)x;
+      bp.a.thr = thr;
+      bp.a.sign = sign;
+      bp.a.y_codes = yc;
+      bp.a.y_acc = ya;
+      bp.a.early = early ? 1 : 0;
+      e = band_dispatch(bp.bn, g.sb, [&](auto inst) { return decltype(inst)::launch(bp, tm, st); });
+    } else {
+      ConvArgs a;
+      fill_conv_args(d, g, bn, x, thr, sign, yc, ya, &a);
+      a.early = early ? 1 : 0;
+      a.wbits = g.in8 ? nullptr : (const uint8_t*)w_prep + prep_pbits_offset(d, g);
+      // Filter tiles expanded from sign bits in shared memory (the split instance only, its TMA warp
+      // streaming the bits): opt-in.  It reads 1 bit per weight from DRAM instead of an e4m3 byte, but
+      // on AlexNet's FC layers (b128) it measured 22.4 / 16.3 us against 20.6 / 16.4 us for FC6 / FC7:
+      // those single-tile launches are bound by the K-stage pipeline's latency, not by the filter
+      // stream.  IFQ_TC_BX = 1 takes it where the filters are read about once (at most two 128-row
+      // tiles), 2 wherever the split instance runs.
+      const bool bx = bx_env != 0 && (bx_env == 2 || ceil_div(g.M, kBM) <= 2) && bn == 64 && ks == 2 && gb == 16 &&
+                      g.sbi == 2 && g.sb == 2;
+      CUtensorMap tm;
+      if (!(bx ? encode_bitmap(d, g, w_prep, bn, &tm) : encode_wmap(d, g, w_prep, bn, &tm))) return IFQ_ECUDA;
+      if (g.sbi == 2 && g.sb == 2) {
+        if (gb == 16) e = launch_tc_gb<16, 2, 2>(bn, ks, tm, a, nsm, st, bx);
+        else if (gb == 8) e = launch_tc_gb<8, 2, 2>(bn, ks, tm, a, nsm, st);
+        else if (gb == 4) e = launch_tc_gb<4, 2, 2>(bn, ks, tm, a, nsm, st);
+        else e = launch_tc_gb<1, 2, 2>(bn, ks, tm, a, nsm, st);
+      } else if (g.sb == 4) {
+        if (gb == 16) e = launch_tc_gb<16, 4, 4>(bn, ks, tm, a, nsm, st);
+        else if (gb == 8) e = launch_tc_gb<8, 4, 4>(bn, ks, tm, a, nsm, st);
+        else e = launch_tc_gb<4, 4, 4>(bn, ks, tm, a, nsm, st);
+      } else {   // 8-bit input values, 2-bit output codes
+        if (gb == 16) e = launch_tc_gb<16, 4, 2>(bn, ks, tm, a, nsm, st);
+        else if (gb == 8) e = launch_tc_gb<8, 4, 2>(bn, ks, tm, a, nsm, st);
+        else e = launch_tc_gb<4, 4, 2>(bn, ks, tm, a, nsm, st);
+      }
     }
   } else if (narrow_supported(d, g)) {
     NarrowArgs a;
@@ -1193,7 +1451,7 @@ int launch_stack_kernel(const ifq_layer* layers, int nlayers, const void* x, voi
     const ifq_layer& l = layers[i];
     ConvGeom g;
     check_conv(&l.conv, &g);
-    const int bn = choose_bn(g, l.conv.cout, nsm);
+    const int bn = choose_bn(g, l.conv.cout, nsm, env_int("IFQ_TC_BN", 0));
     if (!encode_wmap(&l.conv, g, l.w_prep, bn, &P.tm[i])) return IFQ_ECUDA;
     uint8_t* yc = (l.conv.out_mode & IFQ_OUT_CODES) ? (uint8_t*)l.y_codes : nullptr;
     int32_t* ya = (l.conv.out_mode & IFQ_OUT_ACC) ? l.y_acc : nullptr;
@@ -1462,6 +1720,13 @@ int ifq_pack_weights(const ifq_conv_desc* d, const uint32_t* w_bits, void* w_pre
     prep_direct_masks_kernel<<<launch_1d_blocks((size_t)g.K, 256, nsm), 256, 0, S(stream)>>>(
         (const uint32_t*)(base + prep_bits_offset(d, g)), (uint32_t*)(base + prep_masks_offset(d, g)), d->cout, g.K,
         g.kwords);
+  BandGeom bg;
+  if (band_geom(d, g, &bg)) {
+    const long total = (long)bg.cols * bg.crows;
+    prep_band_kernel<<<launch_1d_blocks((size_t)total, 256, nsm), 256, 0, S(stream)>>>(
+        w_bits, (uint4*)(base + prep_band_offset(d, g)), d->cout, bg.crows, g.kwords, bg.fields, bg.dig, bg.taps,
+        bg.npair, total);
+  }
   return cudaGetLastError() == cudaSuccess ? IFQ_OK : IFQ_ECUDA;
 }
 

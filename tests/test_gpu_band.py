@@ -1,0 +1,69 @@
+"""The band kernel (4-bit products on an input band expanded once) on every launch shape of its table, bit-exact
+against the CPU oracle: ragged maps and channel tiles, each load granule (16, 8, 4, 2 and 1 bytes), odd plane
+counts, several chunks and tiles, strided 1 x 1 filters, 2-, 3- and 4-bit codes, and thresholds that saturate or are not
+equally spaced (compared one by one instead of by the fitted line).  The results are integers: no tolerance."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import oracle as O
+from paper_1911_08076_gb300 import ifq, synth
+
+pytestmark = [pytest.mark.gpu,
+              pytest.mark.skipif(not torch.cuda.is_available(), reason="needs a CUDA GPU")]
+
+SHAPES = 6   # launch shapes: IFQ_BAND = 2 .. 7
+CASES = [
+    # n, h, w, cin, cout, k, stride, pad, bits per code
+    (2, 16, 16, 64, 64, 3, 1, 1, 2),      # 16-byte granules, one tile of channels
+    (3, 11, 13, 128, 256, 3, 1, 1, 2),    # several tiles with ragged tails
+    (9, 37, 45, 72, 100, 3, 1, 1, 2),     # 2-byte granules, an odd plane, ragged channels
+    (2, 9, 9, 36, 132, 3, 1, 2, 2),       # 1-byte granules, two channel tiles, the last one ragged
+    (2, 8, 9, 32, 40, 3, 1, 1, 2),        # one plane: taps in pairs, the last alone
+    (2, 12, 12, 16, 36, 3, 1, 1, 2),      # 4-byte granules
+    (1, 27, 27, 96, 64, 5, 1, 2, 2),      # 25 taps, 8-byte granules
+    (4, 7, 7, 512, 192, 3, 1, 1, 2),      # 16 planes in chunks
+    (2, 8, 8, 256, 320, 1, 1, 0, 2),      # 1 x 1 on the map as it lies
+    (3, 15, 14, 64, 72, 1, 2, 0, 2),      # strided 1 x 1
+    (40, 13, 13, 32, 64, 3, 1, 0, 2),     # no padding, many tiles
+    (2, 9, 9, 24, 40, 3, 1, 1, 4),
+    (3, 14, 10, 40, 96, 3, 1, 1, 3),
+    (2, 13, 13, 384, 136, 3, 1, 1, 4),    # 24 planes of digits
+]
+
+
+def _thresholds(rng, cout, K, kbits, even):
+    """Ascending thresholds across the accumulator's spread: floors of equally spaced values, or any."""
+    L = (1 << kbits) - 1
+    sd = np.sqrt(K * L * (2 * L + 1) / 6.0)
+    step, base = rng.uniform(0.3, 1.0, cout) * 3 * sd / L, rng.normal(0, 0.3 * sd, cout)
+    step[1::5] *= 10.0 ** rng.integers(-1, 5, step[1::5].shape)   # steep ones, and thresholds past the bound L K
+    T = np.floor(base[:, None] + step[:, None] * (np.arange(L) - (L - 1) / 2))
+    if not even:
+        T[::3] += np.cumsum(rng.integers(0, int(sd) + 2, T[::3].shape), axis=1)
+    return np.clip(T, -L * K - 1, L * K).astype(np.int32), np.where(rng.integers(0, 4, cout) == 0, -1, 1).astype(np.int8)
+
+
+@pytest.mark.parametrize("case", CASES, ids=[f"c{c[3]}x{c[4]}k{c[5]}s{c[6]}b{c[8]}" for c in CASES])
+def test_every_launch_shape_matches_oracle(case, monkeypatch):
+    n, h, w, cin, cout, k, stride, pad, kbits = case
+    rng = np.random.default_rng(cin * 131 + cout)
+    x = rng.integers(0, 1 << kbits, (n, h, w, cin), dtype=np.uint8)
+    wt = np.where(rng.integers(0, 2, (cout, k, k, cin)) == 1, 1, -1).astype(np.int8)
+    A = O.conv_acc(x, wt, stride, pad)
+    d = ifq.conv_desc(n, h, w, cin, cout, k, stride, pad, ifq.IFQ_OUT_BOTH, ifq.IFQ_PATH_TC, kbits=kbits)
+    xp = torch.from_numpy(synth.pack_codes(x, kbits)).cuda()
+    prep = torch.empty(ifq.ifq_weights_prep_bytes(d), dtype=torch.uint8, device="cuda")
+    ifq.ifq_pack_weights(d, torch.from_numpy(synth.pack_signs(wt).view(np.int32)).cuda(), prep)
+    rowb = cout * synth.field_bits(kbits) // 8
+    for even in (True, False):
+        T, s = _thresholds(rng, cout, k * k * cin, kbits, even)
+        C = O.int_chain(A, T, s)
+        for shape in range(1, 2 + SHAPES):   # 1: the planner's choice
+            monkeypatch.setenv("IFQ_BAND", str(shape))
+            yc = torch.full((*A.shape[:3], rowb), 0x5A, dtype=torch.uint8, device="cuda")
+            ya = torch.full(A.shape, -777777, dtype=torch.int32, device="cuda")
+            ifq.ifq_conv2bit(d, xp, prep, torch.from_numpy(T).cuda(), torch.from_numpy(s).cuda(), yc, ya)
+            assert ifq.ifq_device_status() == ifq.IFQ_OK
+            assert (ya.cpu().numpy() == A).all(), shape
+            assert (synth.unpack_codes(yc.cpu().numpy(), cout, kbits) == C).all(), (shape, even)
