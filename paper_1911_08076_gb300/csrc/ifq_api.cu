@@ -264,6 +264,15 @@ int launch_1d_blocks(size_t items, int threads, int nsm) {
   return b < 1 ? 1 : (int)b;
 }
 
+// Groups of 16 codes that the packing kernels take as vectors (none where a pointer is not aligned for them), and
+// the blocks they run in.
+size_t pack_vectors(const void* codes, const void* packed, size_t n, int sb) {
+  return (uintptr_t)codes % 16 == 0 && (uintptr_t)packed % (2 * sb) == 0 ? n / 16 : 0;
+}
+unsigned pack_blocks(size_t nvec, size_t nbytes, int nsm) {
+  return (unsigned)launch_1d_blocks(nvec ? (nvec + kPackU - 1) / kPackU : nbytes, kPackThreads, nsm);
+}
+
 // Multiply-high divisor for n / d with 0 <= n < 2^31 (d >= 1): shift = ceil(log2 d),
 // mul = floor(2^32 * (2^shift - d) / d) + 1, n / d = (umulhi(n, mul) + n) >> shift.
 FastDiv make_fastdiv(uint32_t d) {
@@ -1902,10 +1911,11 @@ int ifq_pack_codes_kbits(const uint8_t* codes, void* packed, size_t n, int kbits
   if (n == 0) return IFQ_OK;
   int nsm = 0;
   if ((rc = ensure_init(&nsm))) return rc;
-  const size_t nb = n * sb / 8;
-  if (sb == 2) pack_codes_kernel<2><<<launch_1d_blocks(nb, 256, nsm), 256, 0, S(stream)>>>(codes, (uint8_t*)packed, nb);
-  else pack_codes_kernel<4><<<launch_1d_blocks(nb, 256, nsm), 256, 0, S(stream)>>>(codes, (uint8_t*)packed, nb);
-  return cudaGetLastError() == cudaSuccess ? IFQ_OK : IFQ_ECUDA;
+  const size_t nb = n * sb / 8, nv = pack_vectors(codes, packed, n, sb);
+  const dim3 grid(pack_blocks(nv, nb, nsm)), block(kPackThreads);
+  const cudaError_t e = sb == 2 ? launch_k(pack_codes_kernel<2>, grid, block, 0, S(stream), codes, (uint8_t*)packed, nb, nv)
+                                : launch_k(pack_codes_kernel<4>, grid, block, 0, S(stream), codes, (uint8_t*)packed, nb, nv);
+  return e == cudaSuccess ? IFQ_OK : IFQ_ECUDA;
 }
 
 int ifq_unpack_codes_kbits(const void* packed, uint8_t* codes, size_t n, int kbits, void* stream) {
@@ -1915,11 +1925,12 @@ int ifq_unpack_codes_kbits(const void* packed, uint8_t* codes, size_t n, int kbi
   if (n == 0) return IFQ_OK;
   int nsm = 0;
   if ((rc = ensure_init(&nsm))) return rc;
-  const size_t nb = n * sb / 8;
+  const size_t nb = n * sb / 8, nv = pack_vectors(codes, packed, n, sb);
   const uint8_t* p = (const uint8_t*)packed;
-  if (sb == 2) unpack_codes_kernel<2><<<launch_1d_blocks(nb, 256, nsm), 256, 0, S(stream)>>>(p, codes, nb);
-  else unpack_codes_kernel<4><<<launch_1d_blocks(nb, 256, nsm), 256, 0, S(stream)>>>(p, codes, nb);
-  return cudaGetLastError() == cudaSuccess ? IFQ_OK : IFQ_ECUDA;
+  const dim3 grid(pack_blocks(nv, nb, nsm)), block(kPackThreads);
+  const cudaError_t e = sb == 2 ? launch_k(unpack_codes_kernel<2>, grid, block, 0, S(stream), p, codes, nb, nv)
+                                : launch_k(unpack_codes_kernel<4>, grid, block, 0, S(stream), p, codes, nb, nv);
+  return e == cudaSuccess ? IFQ_OK : IFQ_ECUDA;
 }
 
 int ifq_pack_codes(const uint8_t* codes, void* packed, size_t n, void* stream) {
