@@ -155,7 +155,8 @@ __global__ void __launch_bounds__(kConvThreads, 1)
   const uint32_t sBits = sbase + L::offBits;
   uint32_t* tmem_slot = (uint32_t*)(smem + L::offTmem);
 
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);   // known to be uniform: the roles' branches are
   constexpr uint32_t kCols = 512;
   // tile schedule: cluster cid of G takes tiles cid, cid + G, ... (a cluster is one CTA for KS = 1)
   const uint32_t crank = KS > 1 ? cluster_ctarank() : 0u;

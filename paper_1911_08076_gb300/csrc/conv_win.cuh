@@ -199,7 +199,8 @@ __global__ void __launch_bounds__(kWinThreads, 1)
   uint32_t* tmem_slot = (uint32_t*)(smem + oXchg + a.xchg_bytes + kWinTabBytes + 104);
   uint2* win_stash = (uint2*)(smem + oXchg + a.xchg_bytes + kWinTabBytes + 128);   // 32 ballot pairs a warp
 
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);   // known to be uniform: the roles' branches are
   // CTA c takes channel tile c % nct and the band tiles c / nct, c / nct + G / nct, ... of it
   const int ctile = (int)blockIdx.x % a.nct;
   const int first = (int)blockIdx.x / a.nct, step = (int)gridDim.x / a.nct;
