@@ -16,6 +16,7 @@
 #include <vector>
 
 #include "conv_band.cuh"
+#include "conv_march.cuh"
 #include "conv_bitserial.cuh"
 #include "conv_direct.cuh"
 #include "conv_tc.cuh"
@@ -209,9 +210,9 @@ cudaError_t set_warp_attrs() {
   set(set_warp_attr<8, 1, 1, 1>()); set(set_warp_attr<8, 1, 2, 1>());
   set(set_warp_attr<8, 2, 1, 1>()); set(set_warp_attr<8, 2, 2, 1>());
   set(set_warp_attr<8, 4, 1, 1>()); set(set_warp_attr<8, 4, 2, 1>());
-  set(set_warp_attr<8, 1, 1, 0>()); set(set_warp_attr<8, 1, 2, 0>());
-  set(set_warp_attr<8, 2, 1, 0>()); set(set_warp_attr<8, 2, 2, 0>());
-  set(set_warp_attr<8, 4, 1, 0>()); set(set_warp_attr<8, 4, 2, 0>());
+  set(set_warp_attr<8, 1, 1, 0>());
+  set(set_warp_attr<8, 2, 1, 0>());
+  set(set_warp_attr<8, 4, 1, 0>());
   set(set_warp_attr<16, 1, 1, 0>()); set(set_warp_attr<16, 1, 2, 0>());
   set(set_warp_attr<16, 2, 1, 0>()); set(set_warp_attr<16, 2, 2, 0>());
   set(set_warp_attr<16, 4, 1, 0>()); set(set_warp_attr<16, 4, 2, 0>());
@@ -619,7 +620,10 @@ cudaError_t launch_warp_en(int pool, bool in8, int nsm, size_t smem, cudaStream_
     if (in8)
       return pool == 2 ? launch_warp_inst<E, NT, 2, 1>(nsm, smem, st, a) : launch_warp_inst<E, NT, 1, 1>(nsm, smem, st, a);
   }
-  return pool == 2 ? launch_warp_inst<E, NT, 2, 0>(nsm, smem, st, a) : launch_warp_inst<E, NT, 1, 0>(nsm, smem, st, a);
+  if constexpr (E == 16) {   // (8 channels of codes under a pool: the march kernel)
+    if (pool == 2) return launch_warp_inst<E, NT, 2, 0>(nsm, smem, st, a);
+  }
+  return launch_warp_inst<E, NT, 1, 0>(nsm, smem, st, a);
 }
 
 cudaError_t launch_warp(int E, int NT, int pool, bool in8, int nsm, size_t smem, cudaStream_t st,
@@ -631,6 +635,41 @@ cudaError_t launch_warp(int E, int NT, int pool, bool in8, int nsm, size_t smem,
   return NT == 1 ? launch_warp_en<16, 1>(pool, false, nsm, smem, st, a)
                  : (NT == 2 ? launch_warp_en<16, 2>(pool, false, nsm, smem, st, a)
                             : launch_warp_en<16, 4>(pool, false, nsm, smem, st, a));
+}
+
+// The march kernel (conv_march.cuh): 3 x 3, stride 1, a fused 2 x 2 pool, 2-bit codes out, 4 channels of 8-bit
+// values or 8 of 2-bit codes in.  It takes the layers of this form of the direct path (up to 16 channels: 45 against
+// 65 us on 4 -> 8 at 416 x 416, batch 64) and of the warp path (32 against 42 us on 8 -> 16 at 208 x 208).
+bool march_supported(const ifq_conv_desc* d, const ConvGeom& g) {
+  return g.pool == 2 && d->kh == 3 && d->kw == 3 && d->stride == 1 && g.sb == 2 && g.lvl == 3 && d->cout % 4 == 0 &&
+         (g.in8 ? d->cin == 4 && d->cout <= 16 : g.kb == 2 && d->cin == 8 && d->cout <= 32);
+}
+
+cudaError_t launch_march(const ifq_conv_desc* d, const ConvGeom& g, int nsm, const void* x, const void* w_prep,
+                         const int32_t* thr, const int8_t* sign, uint8_t* y, cudaStream_t st) {
+  MarchArgs a;
+  a.x = x;
+  a.w = (const uint32_t*)((const uint8_t*)w_prep + (g.in8 ? prep_masks_offset(d, g) : prep_bits_offset(d, g)));
+  a.thr = thr;
+  a.sign = sign;
+  a.y = y;
+  a.h = d->h; a.w_in = d->w; a.cout = d->cout; a.kwords = g.kwords; a.pad = d->pad; a.pho = g.pho; a.pwo = g.pwo;
+  // a warp loads its weights and the first rows of a march once: long marches, while every SM has its warps
+  const int strips = ceil_div(g.pwo, 8), per_sm = 8;
+  a.ry = 16;
+  while (a.ry > 2 && (long long)d->n * strips * ceil_div(g.pho, a.ry) < (long long)nsm * per_sm * (kMarchThreads / 32))
+    a.ry /= 2;
+  const int blocks = ceil_div(g.pho, a.ry);
+  a.units = d->n * strips * blocks;
+  a.div_strips = make_fastdiv((uint32_t)strips);
+  a.div_blocks = make_fastdiv((uint32_t)blocks);
+  const dim3 grid((unsigned)std::min(ceil_div(a.units, kMarchThreads / 32), nsm * per_sm)), block(kMarchThreads);
+  if (g.in8)
+    return d->cout <= 8 ? launch_k(conv_march_kernel<1, 1>, grid, block, 0, st, a)
+                        : launch_k(conv_march_kernel<1, 2>, grid, block, 0, st, a);
+  return d->cout <= 8 ? launch_k(conv_march_kernel<0, 1>, grid, block, 0, st, a)
+                      : (d->cout <= 16 ? launch_k(conv_march_kernel<0, 2>, grid, block, 0, st, a)
+                                       : launch_k(conv_march_kernel<0, 4>, grid, block, 0, st, a));
 }
 
 int choose_path(const ifq_conv_desc* d, const ConvGeom& g) {
@@ -1029,7 +1068,9 @@ int run_conv(const ifq_conv_desc* d, const void* x, const void* w_prep, const in
   const int path = choose_path(d, g);
   if (path < 0) return IFQ_EUNSUPPORTED;
   cudaError_t e;
-  if (path == IFQ_PATH_DIRECT) {
+  if ((path == IFQ_PATH_DIRECT || (path == IFQ_PATH_WARP && !g.in8)) && march_supported(d, g)) {
+    e = launch_march(d, g, nsm, x, w_prep, thr, sign, yc, st);
+  } else if (path == IFQ_PATH_DIRECT) {
     DirectArgs a;
     a.x = (const uint8_t*)x;
     a.wmask = (const uint32_t*)((const uint8_t*)w_prep + prep_masks_offset(d, g));
