@@ -13,17 +13,21 @@
 // moved into f16 halves by a permute or a mask.  The bits are read as f16 subnormals, x * 2^-24 (a field 4^i x
 // against a weight of 4^-i), so no conversion is needed, and every product and fp32 sum is an exact integer
 // multiple of 2^-24.  A pixel is loaded and expanded once per filter column and window column and kept over the
-// rows of the march; the next rows are loaded a step ahead.
+// rows of the march; the rows are loaded two steps ahead.
 //
 // Measured (us, batch 64, pooled; the kernel before, this one): 3 x 3 4 -> 8 on 416 x 416 8-bit pixels 64.9 (dp4a, the
-// direct kernel), 45.1; 3 x 3 8 -> 16 on 208 x 208 2-bit codes 41.9 (the warp kernel's e4m3 mma.sync, which
-// issues as four instructions), 32.3.  Their bytes take 7.5 and 2.5 us: issue slots and the f16 pipe bound both.
+// direct kernel), 43.9; 3 x 3 8 -> 16 on 208 x 208 2-bit codes 41.9 (the warp kernel's e4m3 mma.sync, which
+// issues as four instructions), 30.3.  Their bytes take 7.5 and 2.5 us: instructions and the latency of
+// loads and products bound both (issue slots 37 and 49 % busy; rows loaded one step ahead 45.2 and 32.3).
 #pragma once
 #include "conv_common.cuh"
 
 namespace ifq {
 
 constexpr int kMarchThreads = 128;
+
+// CTAs per SM: as many as their registers allow.
+__host__ __device__ constexpr int march_ctas(int in8, int nt) { return in8 ? (nt == 1 ? 8 : 5) : (nt == 1 ? 5 : (nt == 2 ? 4 : 3)); }
 
 struct MarchArgs {
   const void* x;           // 8-bit values, 4 a pixel, or 2-bit codes, 8 a pixel
@@ -46,7 +50,7 @@ __device__ __forceinline__ void mma_f16(float (&d)[4], uint32_t a0, uint32_t a1,
 
 // IN8: 1 for 8-bit values; NT: tiles of 8 output channels.
 template <int IN8, int NT>
-__global__ void __launch_bounds__(kMarchThreads) conv_march_kernel(const MarchArgs a) {
+__global__ void __launch_bounds__(kMarchThreads, march_ctas(IN8, NT)) conv_march_kernel(const MarchArgs a) {
   constexpr int NR = IN8 ? 2 : 4;                    // f16 pairs of a pixel
   constexpr int KS = NR / 2;                         // K steps of a filter row
   using Word = typename std::conditional<IN8 != 0, uint32_t, uint16_t>::type;
@@ -103,8 +107,8 @@ __global__ void __launch_bounds__(kMarchThreads) conv_march_kernel(const MarchAr
     const bool c0 = t < 3 && (unsigned)ix < (unsigned)w, c1 = t < 3 && (unsigned)(ix + 1) < (unsigned)w;
     int iy = 2 * y0 - a.pad;                         // the next input row
     const Word* p = (const Word*)a.x + ((long long)img * a.h + iy) * w + ix;
-    uint32_t raw[2][2];
-    auto load = [&]() {                              // two input rows, window columns 0 and 1
+    uint32_t qa[2][2], qb[2][2];                     // the pixels of the next two row pairs, in turn
+    auto load = [&](uint32_t (&raw)[2][2]) {                              // two input rows, window columns 0 and 1
 #pragma unroll
       for (int r = 0; r < 2; ++r, ++iy, p += w) {
         const bool ok = (unsigned)iy < (unsigned)a.h;
@@ -113,7 +117,7 @@ __global__ void __launch_bounds__(kMarchThreads) conv_march_kernel(const MarchAr
       }
     };
     uint32_t ra[2][2][NR], rb[2][2][NR];             // rows 0, 1 and 2, 3 of the window, in turn
-    auto expand = [&](uint32_t (&v)[2][2][NR]) {
+    auto expand = [&](const uint32_t (&raw)[2][2], uint32_t (&v)[2][2][NR]) {
 #pragma unroll
       for (int r = 0; r < 2; ++r)
 #pragma unroll
@@ -130,9 +134,9 @@ __global__ void __launch_bounds__(kMarchThreads) conv_march_kernel(const MarchAr
     };
     uint8_t* dst = a.y + ((size_t)((size_t)img * a.pho + y0) * a.pwo + X) * rowb;
     // one pooled row: `top` the first two input rows, the next two expanded into `bot`
-    auto row = [&](const uint32_t (&top)[2][2][NR], uint32_t (&bot)[2][2][NR], bool more) {
-      expand(bot);
-      if (more) load();
+    auto row = [&](const uint32_t (&top)[2][2][NR], uint32_t (&bot)[2][2][NR], uint32_t (&raw)[2][2], bool more) {
+      expand(raw, bot);
+      if (more) load(raw);
       float d[2][NT][4];
 #pragma unroll
       for (int py = 0; py < 2; ++py)
@@ -176,13 +180,14 @@ __global__ void __launch_bounds__(kMarchThreads) conv_march_kernel(const MarchAr
       }
       dst += (size_t)a.pwo * rowb;
     };
-    load();
-    expand(ra);
-    load();
+    load(qb);
+    load(qa);
+    expand(qb, ra);
+    load(qb);
 #pragma unroll 1
     for (int y = 0; y < ny; y += 2) {
-      row(ra, rb, y + 1 < ny);
-      if (y + 1 < ny) row(rb, ra, y + 2 < ny);
+      row(ra, rb, qa, y + 2 < ny);
+      if (y + 1 < ny) row(rb, ra, qb, y + 3 < ny);
     }
   }
 }

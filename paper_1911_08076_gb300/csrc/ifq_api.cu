@@ -638,8 +638,8 @@ cudaError_t launch_warp(int E, int NT, int pool, bool in8, int nsm, size_t smem,
 }
 
 // The march kernel (conv_march.cuh): 3 x 3, stride 1, a fused 2 x 2 pool, 2-bit codes out, 4 channels of 8-bit
-// values or 8 of 2-bit codes in.  It takes the layers of this form of the direct path (up to 16 channels: 45 against
-// 65 us on 4 -> 8 at 416 x 416, batch 64) and of the warp path (32 against 42 us on 8 -> 16 at 208 x 208).
+// values or 8 of 2-bit codes in.  It takes the layers of this form of the direct path (up to 16 channels: 44 against
+// 65 us on 4 -> 8 at 416 x 416, batch 64) and of the warp path (30 against 42 us on 8 -> 16 at 208 x 208).
 bool march_supported(const ifq_conv_desc* d, const ConvGeom& g) {
   return g.pool == 2 && d->kh == 3 && d->kw == 3 && d->stride == 1 && g.sb == 2 && g.lvl == 3 && d->cout % 4 == 0 &&
          (g.in8 ? d->cin == 4 && d->cout <= 16 : g.kb == 2 && d->cin == 8 && d->cout <= 32);
@@ -654,11 +654,19 @@ cudaError_t launch_march(const ifq_conv_desc* d, const ConvGeom& g, int nsm, con
   a.sign = sign;
   a.y = y;
   a.h = d->h; a.w_in = d->w; a.cout = d->cout; a.kwords = g.kwords; a.pad = d->pad; a.pho = g.pho; a.pwo = g.pwo;
-  // a warp loads its weights and the first rows of a march once: long marches, while every SM has its warps
-  const int strips = ceil_div(g.pwo, 8), per_sm = 8;
-  a.ry = 16;
-  while (a.ry > 2 && (long long)d->n * strips * ceil_div(g.pho, a.ry) < (long long)nsm * per_sm * (kMarchThreads / 32))
-    a.ry /= 2;
+  // The rows of a march: the smallest number of steps until the last warp is done.  A march costs about four
+  // steps more than its rows (its first loads; 16 rows for every layer left a ragged last round).
+  const int strips = ceil_div(g.pwo, 8), nt = ceil_div(d->cout, 8), per_sm = march_ctas(g.in8 ? 1 : 0, nt);
+  const long long warps = (long long)nsm * per_sm * (kMarchThreads / 32);
+  long long best = 0;
+  for (int ry = 1; ry <= 32; ++ry) {
+    const long long units = (long long)d->n * strips * ceil_div(g.pho, ry);
+    const long long steps = (units + warps - 1) / warps * (ry + 4);
+    if (best == 0 || steps < best) {
+      best = steps;
+      a.ry = ry;
+    }
+  }
   const int blocks = ceil_div(g.pho, a.ry);
   a.units = d->n * strips * blocks;
   a.div_strips = make_fastdiv((uint32_t)strips);
