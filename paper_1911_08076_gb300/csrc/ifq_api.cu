@@ -2,6 +2,8 @@
 // quantized convolution (tensor-core and bit-serial paths), code pooling,
 // the layer-stack driver and its CUDA-graph form, packing helpers and the
 // device status word.  Host-only calls (the fold, shapes) live in ifq_host.cpp.
+#include <unistd.h>
+
 #include <cuda.h>
 #include <cuda_runtime.h>
 #include <cudaTypedefs.h>
@@ -286,7 +288,22 @@ FastDiv make_fastdiv(uint32_t d) {
   return f;
 }
 
+// Within an EnvScope a thread looks once whether the environment holds any of the library's switches; where it holds
+// none, env_int answers without a search (a convolution asks for seven, about 0.1 us each).
+thread_local bool t_no_switches = false;
+
+struct EnvScope {
+  const bool outer = t_no_switches;
+  EnvScope() {
+    bool any = false;
+    for (char** e = environ; e && *e && !any; ++e) any = (*e)[0] == 'I' && strncmp(*e, "IFQ_", 4) == 0;
+    t_no_switches = !any;
+  }
+  ~EnvScope() { t_no_switches = outer; }
+};
+
 int env_int(const char* name, int dflt) {
+  if (t_no_switches) return dflt;
   const char* v = getenv(name);
   return (v && *v) ? atoi(v) : dflt;
 }
@@ -1060,6 +1077,7 @@ double tc_cycles(const ConvGeom& g, int cout, int nsm, int bn, int ks, int gb, b
 // stack after the first), so the tensor-core kernel may load them before its dependency wait.
 int run_conv(const ifq_conv_desc* d, const void* x, const void* w_prep, const int32_t* thr, const int8_t* sign,
              void* y_codes, int32_t* y_acc, cudaStream_t st, bool early = false) {
+  const EnvScope env;
   ConvGeom g;
   int rc = check_conv(d, &g);
   if (rc) return rc;

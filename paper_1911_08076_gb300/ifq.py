@@ -105,6 +105,8 @@ def lib_path() -> str:
 def lib(build_if_missing: bool = True):
     """The loaded libifq.so (built in-tree on first use if missing)."""
     global _lib
+    if _lib is not None:
+        return _lib
     with _lock:
         if _lib is None:
             try:  # let torch load its CUDA runtime first so one libcudart serves both
@@ -136,7 +138,8 @@ def _ptr(t) -> Optional[int]:
 def _stream(stream) -> Optional[int]:
     if stream is None:
         import torch
-        return torch.cuda.current_stream().cuda_stream
+        # (the handle without a Stream object around it)
+        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
     if isinstance(stream, int):
         return stream
     return stream.cuda_stream
