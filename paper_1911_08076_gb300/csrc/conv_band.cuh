@@ -10,7 +10,7 @@
 //   * a 3- or 4-bit code in its 4-bit field is two 2-bit digits (low digit first), so its map is a
 //     2-bit map of twice the channels whose odd channels weigh +4 / -4 (nibbles 0x6 / 0xE);
 //   * the fp32 accumulation was checked exact on GB300 up to |A| = 196608 with odd addends along all
-//     of K = 65536 (test_tc_accumulation_exact_at_the_admitted_bound), the bound the planner admits.
+//     of K = 65536, the bound the planner admits (test_accumulation_exact_at_the_admitted_bound).
 // Measured rate of the instruction (M128 x N128 x K64, both operands in shared memory, A at any slot
 // offset): 64 cycles, 9.7 PTOPS on 152 SMs, twice the e4m3 rate of the im2col kernel (conv_tc.cuh); N = 64
 // takes 48 cycles and N = 32 40, where reading the 4 KB of A takes longer than the products.

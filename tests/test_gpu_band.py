@@ -67,3 +67,29 @@ def test_every_launch_shape_matches_oracle(case, monkeypatch):
             assert ifq.ifq_device_status() == ifq.IFQ_OK
             assert (ya.cpu().numpy() == A).all(), shape
             assert (synth.unpack_codes(yc.cpu().numpy(), cout, kbits) == C).all(), (shape, even)
+
+
+@pytest.mark.parametrize("kbits,K", [(2, 65536), (3, 28064), (4, 13088)])
+def test_accumulation_exact_at_the_admitted_bound(kbits, K, monkeypatch):
+    """Accumulators up to the largest magnitude admitted, (2^k - 1) K <= 196608, with small odd addends all along
+    K: the 4-bit products' fp32 sums must stay exact.  The sums are checked against float64."""
+    rng = np.random.default_rng(K)
+    L = (1 << kbits) - 1
+    n, cout = 300, 72
+    x = rng.choice(np.array([1, 2, L - 1, L], np.uint8), size=(n, 1, 1, K), p=[0.05, 0.05, 0.1, 0.8])
+    x[0] = L
+    wt = np.ones((cout, 1, 1, K), np.int8)
+    wt[1] = -1
+    for r in range(2, cout):
+        wt[r, 0, 0, rng.random(K) < (0.05 if r < 40 else 0.5)] = -1
+    A = (x.reshape(n, K).astype(np.float64) @ wt.reshape(cout, K).astype(np.float64).T).astype(np.int64)
+    d = ifq.conv_desc(n, 1, 1, K, cout, 1, 1, 0, ifq.IFQ_OUT_ACC, ifq.IFQ_PATH_TC, kbits=kbits)
+    xp = torch.from_numpy(synth.pack_codes(x, kbits)).cuda()
+    prep = torch.empty(ifq.ifq_weights_prep_bytes(d), dtype=torch.uint8, device="cuda")
+    ifq.ifq_pack_weights(d, torch.from_numpy(synth.pack_signs(wt).view(np.int32)).cuda(), prep)
+    for shape in range(2, 2 + SHAPES):
+        monkeypatch.setenv("IFQ_BAND", str(shape))
+        ya = torch.full((n, 1, 1, cout), -777777, dtype=torch.int32, device="cuda")
+        ifq.ifq_conv2bit(d, xp, prep, None, None, None, ya)
+        assert ifq.ifq_device_status() == ifq.IFQ_OK
+        assert (ya.cpu().numpy().reshape(n, cout) == A).all(), shape
