@@ -52,7 +52,8 @@
 // Measured (us; im2col kernel, this one): 3x3 256 -> 256 on 56 x 56 x 256 images 300, 167 (5.7 PTOPS; 59 % of the
 // instruction's rate); 1x1 512 -> 512 on 28 x 28 x 256 94.7, 43.3; 5x5 96 -> 256 on 27 x 27 x 128 43.5, 25.0; 3x3 1024
 // -> 1024 on 13 x 13 x 64 68.7, 42.8; the same AlexNet 5x5 layer with 4-bit codes 66.1, 47.5.  What bounds the large
-// layers now is issue slots (50 to 59 % busy): the MMA warps' instructions compete with the epilogue's.
+// layers now is instruction latency beside 24 warps (issue slots 48 to 60 % busy): the MMA warps wait for slots that
+// the epilogue takes.
 #pragma once
 #include "conv_common.cuh"
 
