@@ -231,8 +231,9 @@ int ifq_pack_weights(const ifq_conv_desc* d, const uint32_t* w_bits, void* w_pre
 /*
  * The kernel path ifq_conv2bit takes for `d` (host; reads IFQ_FORCE_PATH as
  * ifq_conv2bit does): IFQ_PATH_TC, IFQ_PATH_BITSERIAL, IFQ_PATH_DIRECT,
- * IFQ_PATH_WIN or IFQ_PATH_WARP.  The warp-MMA path (mma.sync e4m3 tiles of
- * 16 pixels x 8 channels, accumulators and the fused pool in registers)
+ * IFQ_PATH_WIN or IFQ_PATH_WARP.  The warp-MMA path (mma.sync tiles of 16 pixels x 8
+ * channels, e4m3 or, with 8 channels of codes and a fused pool, f16; accumulators and the
+ * fused pool in registers)
  * serves 3 x 3 stride-1 layers with padding 1 on 2-bit codes with cin 8 or 16
  * or on 8-bit values with cin 4, with 2-bit codes or accumulators out,
  * cout 8, 16 or 32, and no pool or a 2 x 2 pool on even sizes; it is the
@@ -247,10 +248,13 @@ int ifq_pack_weights(const ifq_conv_desc* d, const uint32_t* w_bits, void* w_pre
  * measured faster), and a request for it elsewhere takes the tensor-core
  * path.  The
  * tensor-core path needs (2^k - 1)*K <= 196608 (the accumulator range checked
- * exact on the fp8 tensor cores; 255*K for 8-bit inputs), kh, kw <= 15, and
- * for k = 3, 4 cin % 8 == 0; a request for it outside that range takes the
+ * exact on the fp8 and fp4 tensor cores; 255*K for 8-bit inputs), kh, kw <= 15, and
+ * for k = 3, 4 cin % 8 == 0; it runs an im2col kernel or, for unpooled layers on
+ * codes with stride 1 or a 1 x 1 filter and more than 32 channels where that is estimated faster,
+ * a band kernel; a request for it outside that range takes the
  * bit-serial path.  The direct CUDA-core path serves layers on 8-bit inputs
- * with cout <= 32 and K <= 257 (the default for them); a request for it
+ * with cout <= 32 and K <= 257 (the default for them; 3 x 3 layers with cin 4, cout <= 16,
+ * 2-bit codes out and a fused 2 x 2 pool run on f16 mma.sync instead); a request for it
  * elsewhere takes the tensor-core path.  IFQ_EUNSUPPORTED for a fused pool
  * or an 8-bit input that would land on the bit-serial path.
  */
