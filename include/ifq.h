@@ -215,7 +215,16 @@ int ifq_conv_out_shape(const ifq_conv_desc* d, int* ho, int* wo);   /* after the
 
 /*
  * Size of the prepared-filter buffer that ifq_pack_weights fills for `d`
- * (host, pure).  The prepared layout is private to the library.
+ * (host, pure).  The prepared layout is private to the library and may change
+ * with ifq_version.  Layout and size depend on cin, cout, kh, kw and the
+ * stored field width (in_bits 8, or 2- or 4-bit fields) alone: filters
+ * prepared for one descriptor serve every descriptor that agrees in these,
+ * whatever its map, stride, padding, pool, outputs or path.  With more than
+ * 32 output channels, kh, kw <= 15 and at most 49 taps (and, in 4-bit fields,
+ * cin % 8 == 0 and 7*K <= 196608) codes are served by two tensor-core kernels,
+ * and the buffer holds the operands of both: per weight 1 byte and two sign
+ * bits, and 1/2 byte (2-bit fields) or 1 byte (4-bit fields) more for the band
+ * kernel, also where a layer with these filters runs on another path.
  */
 int ifq_weights_prep_bytes(const ifq_conv_desc* d, size_t* bytes);
 
@@ -271,7 +280,7 @@ int ifq_conv_workspace_bytes(const ifq_conv_desc* d, size_t* bytes);
  *   y_codes = #{ i : sign[n]*A > thr[n][i] }  (k-bit codes, packed)
  *   y_acc   = A                                (int32), per out_mode
  * x (device): packed codes; w_prep (device): from ifq_pack_weights for the
- * same descriptor; thr (device): int32 [cout][2^k - 1], ascending per channel;
+ * same filters (see ifq_weights_prep_bytes); thr (device): int32 [cout][2^k - 1], ascending per channel;
  * sign (device): int8 [cout];
  * y_codes (device, out_mode & CODES): packed [n][ho][wo][cout*f/8] bytes;
  * y_acc (device, out_mode & ACC): int32 [n][ho][wo][cout];

@@ -375,22 +375,20 @@ size_t prep_masks_offset(const ifq_conv_desc* d, const ConvGeom& g) {
 // 8-bit-input layers keep their masks.
 size_t prep_pbits_offset(const ifq_conv_desc* d, const ConvGeom& g) { return prep_masks_offset(d, g); }
 
-// Geometry of the band path (conv_band.cuh) that depends on the layer alone, or false where the path does
-// not apply.  It takes 2-, 3- or 4-bit codes without a fused pool, stride 1 or a 1 x 1 filter, at most
-// kBandMaxTaps filter taps, more than 32 output channels and an accumulator magnitude inside the checked exact
-// range.  Filters that cover their whole unpadded input (fully connected layers) are left out: a 6 x 6 x 256 ->
-// 4096 layer at batch 128 measured 30.5 us here (as a 1 x 1 layer on the flattened input) against 13.7 us on
-// the im2col kernel, which splits K.
+// The band path's prepared filters (conv_band.cuh), or false where a layer has none.  Like the rest of the prepared
+// layout this depends on the filters and the stored width of the codes alone, never on the map, stride, padding,
+// pool, outputs or path of a descriptor, nor on which of the two code widths of a 4-bit field it says: filters
+// prepared once serve every layer that uses them.  More than 32 output channels, at most kBandMaxTaps taps, and
+// what else the tensor-core path asks of the filters.
 struct BandGeom {
   int fields, dig;                            // 2-bit fields per pixel, digits per code
   int taps, planes, npair, nodd, cols, crows;
 };
 
-bool band_geom(const ifq_conv_desc* d, const ConvGeom& g, BandGeom* b) {
-  if (g.in8 || g.pool != 1 || d->cout <= 32 || (long long)g.lvl * g.K > kTcMaxAcc) return false;
+bool band_filters(const ifq_conv_desc* d, const ConvGeom& g, BandGeom* b) {
+  if (g.in8 || d->cout <= 32 || d->kh > 15 || d->kw > 15 || d->kh * d->kw > kBandMaxTaps) return false;
+  if (g.sb == 4 && (d->cin % 8 != 0 || 7LL * g.K > kTcMaxAcc)) return false;   // (7: the fewer levels of the two)
   b->taps = d->kh * d->kw;
-  if (b->taps > kBandMaxTaps || (d->stride != 1 && b->taps != 1)) return false;
-  if (b->taps > 1 && d->pad == 0 && d->kh == d->h && d->kw == d->w) return false;
   b->dig = g.sb / 2;
   b->fields = d->cin * b->dig;
   b->planes = ceil_div(b->fields, 32);
@@ -401,6 +399,16 @@ bool band_geom(const ifq_conv_desc* d, const ConvGeom& g, BandGeom* b) {
   return true;
 }
 
+// Whether the band path takes a layer: no fused pool, stride 1 or a 1 x 1 filter, and an accumulator magnitude
+// inside the checked exact range.  Filters that cover their whole unpadded input (fully connected layers) are left
+// out: a 6 x 6 x 256 -> 4096 layer at batch 128 measured 30.5 us here (as a 1 x 1 layer on the flattened input)
+// against 13.7 us on the im2col kernel, which splits K.
+bool band_geom(const ifq_conv_desc* d, const ConvGeom& g, BandGeom* b) {
+  if (!band_filters(d, g, b) || g.pool != 1 || (long long)g.lvl * g.K > kTcMaxAcc) return false;
+  if (d->stride != 1 && b->taps != 1) return false;
+  return !(b->taps > 1 && d->pad == 0 && d->kh == d->h && d->kw == d->w);
+}
+
 // Layers on codes: then the band path's filters, [core column][cout][16 bytes].
 size_t prep_band_offset(const ifq_conv_desc* d, const ConvGeom& g) {
   return round_up(prep_pbits_offset(d, g) + (size_t)d->cout * g.Kpad / 8, 256);
@@ -409,7 +417,7 @@ size_t prep_band_offset(const ifq_conv_desc* d, const ConvGeom& g) {
 size_t prep_bytes(const ifq_conv_desc* d, const ConvGeom& g) {
   if (g.in8) return prep_masks_offset(d, g) + (size_t)g.K * 4;
   BandGeom b;
-  if (!band_geom(d, g, &b)) return prep_pbits_offset(d, g) + (size_t)d->cout * g.Kpad / 8;
+  if (!band_filters(d, g, &b)) return prep_pbits_offset(d, g) + (size_t)d->cout * g.Kpad / 8;
   return prep_band_offset(d, g) + (size_t)b.cols * b.crows * 16;
 }
 
@@ -881,7 +889,7 @@ int band_pitch(int out, int in, int k, int s, int pad) {
 // filter rows x 8 core columns (one filter stage), no swizzle.
 bool encode_bandmap(const ifq_conv_desc* d, const ConvGeom& g, const void* w_prep, int bn, CUtensorMap* tm) {
   BandGeom b;
-  if (!get_encode() || !band_geom(d, g, &b)) return false;
+  if (!get_encode() || !band_filters(d, g, &b)) return false;
   cuuint64_t gdim[2] = {(cuuint64_t)b.crows * 2, (cuuint64_t)b.cols};
   cuuint64_t gstride[1] = {(cuuint64_t)b.crows * 16};
   cuuint32_t box[2] = {(cuuint32_t)bn * 2, 8};
@@ -1797,7 +1805,7 @@ int ifq_pack_weights(const ifq_conv_desc* d, const uint32_t* w_bits, void* w_pre
         (const uint32_t*)(base + prep_bits_offset(d, g)), (uint32_t*)(base + prep_masks_offset(d, g)), d->cout, g.K,
         g.kwords);
   BandGeom bg;
-  if (band_geom(d, g, &bg)) {
+  if (band_filters(d, g, &bg)) {
     const long total = (long)bg.cols * bg.crows;
     prep_band_kernel<<<launch_1d_blocks((size_t)total, 256, nsm), 256, 0, S(stream)>>>(
         w_bits, (uint4*)(base + prep_band_offset(d, g)), d->cout, bg.crows, g.kwords, bg.fields, bg.dig, bg.taps,

@@ -358,3 +358,28 @@ def test_warp_path_plan():
             del os.environ["IFQ_WARP"]
         else:
             os.environ["IFQ_WARP"] = old
+
+
+@pytest.mark.parametrize("kbits", [2, 3, 4])
+@pytest.mark.parametrize("cin,cout,k", [(256, 256, 3), (64, 40, 5), (512, 512, 1), (256, 512, 6), (24, 32, 3),
+                                        (1640, 64, 3), (3000, 72, 3), (16, 64, 9)])
+def test_prepared_filters_depend_on_the_filters_alone(cin, cout, k, kbits):
+    """Filters are prepared once and serve every layer that uses them: the buffer's size is the same for any map, stride,
+    padding, fused pool, outputs and path, and for 3- and 4-bit codes, which share a field width."""
+    K = k * k * cin
+    want = None
+    for n, h, w in ((1, k, k), (3, 14, 18)):
+        for stride in (1, 2):
+            for pad in (0, k // 2):
+                for kb in ((2,) if kbits == 2 else (3, 4)):
+                    for pool, mode in ((0, ifq.IFQ_OUT_CODES), (0, ifq.IFQ_OUT_BOTH), (2, ifq.IFQ_OUT_CODES)):
+                        for path in (ifq.IFQ_PATH_AUTO, ifq.IFQ_PATH_TC, ifq.IFQ_PATH_BITSERIAL):
+                            d = ifq.conv_desc(n, h, w, cin, cout, k, stride, pad, mode, path, pool=pool, kbits=kb)
+                            try:
+                                got = ifq.ifq_weights_prep_bytes(d)
+                            except ifq.IfqError as e:   # (a pool over an odd map)
+                                assert pool and e.status == ifq.IFQ_ESHAPE
+                                continue
+                            assert want in (None, got), (n, h, w, stride, pad, kb, pool, mode, path)
+                            want = got
+    assert want >= cout * K

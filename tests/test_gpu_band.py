@@ -93,3 +93,26 @@ def test_accumulation_exact_at_the_admitted_bound(kbits, K, monkeypatch):
         ifq.ifq_conv2bit(d, xp, prep, None, None, None, ya)
         assert ifq.ifq_device_status() == ifq.IFQ_OK
         assert (ya.cpu().numpy().reshape(n, cout) == A).all(), shape
+
+
+@pytest.mark.parametrize("kbits", [2, 4])
+@pytest.mark.parametrize("prepared", ["pooled", "strided", "fully connected", "bit-serial"])
+def test_filters_prepared_for_another_layer_with_them(prepared, kbits, monkeypatch):
+    """Filters prepared from a descriptor that the band kernel does not serve run on it from one that it does."""
+    n, h, w, cin, cout, k = 3, 12, 14, 64, 72, 3
+    rng = np.random.default_rng(7)
+    x = rng.integers(0, 1 << kbits, (n, h, w, cin), dtype=np.uint8)
+    wt = np.where(rng.integers(0, 2, (cout, k, k, cin)) == 1, 1, -1).astype(np.int8)
+    dp = {"pooled": ifq.conv_desc(1, h, w, cin, cout, k, 1, 1, pool=2, kbits=kbits),
+          "strided": ifq.conv_desc(1, h, w, cin, cout, k, 2, 1, kbits=kbits),
+          "fully connected": ifq.conv_desc(1, k, k, cin, cout, k, 1, 0, kbits=kbits),
+          "bit-serial": ifq.conv_desc(1, h, w, cin, cout, k, 3, 1, path=ifq.IFQ_PATH_BITSERIAL, kbits=kbits)}[prepared]
+    d = ifq.conv_desc(n, h, w, cin, cout, k, 1, 1, ifq.IFQ_OUT_ACC, ifq.IFQ_PATH_TC, kbits=kbits)
+    assert ifq.ifq_weights_prep_bytes(dp) == ifq.ifq_weights_prep_bytes(d)
+    prep = torch.empty(ifq.ifq_weights_prep_bytes(dp), dtype=torch.uint8, device="cuda")
+    ifq.ifq_pack_weights(dp, torch.from_numpy(synth.pack_signs(wt).view(np.int32)).cuda(), prep)
+    monkeypatch.setenv("IFQ_BAND", "2")
+    ya = torch.full((n, h, w, cout), -777777, dtype=torch.int32, device="cuda")
+    ifq.ifq_conv2bit(d, torch.from_numpy(synth.pack_codes(x, kbits)).cuda(), prep, None, None, None, ya)
+    assert ifq.ifq_device_status() == ifq.IFQ_OK
+    assert (ya.cpu().numpy() == O.conv_acc(x, wt, 1, 1)).all()
