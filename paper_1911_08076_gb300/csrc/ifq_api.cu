@@ -2,8 +2,6 @@
 // quantized convolution (tensor-core and bit-serial paths), code pooling,
 // the layer-stack driver and its CUDA-graph form, packing helpers and the
 // device status word.  Host-only calls (the fold, shapes) live in ifq_host.cpp.
-#include <unistd.h>
-
 #include <cuda.h>
 #include <cuda_runtime.h>
 #include <cudaTypedefs.h>
@@ -288,22 +286,9 @@ FastDiv make_fastdiv(uint32_t d) {
   return f;
 }
 
-// Within an EnvScope a thread looks once whether the environment holds any of the library's switches; where it holds
-// none, env_int answers without a search (a convolution asks for seven, about 0.1 us each).
-thread_local bool t_no_switches = false;
-
-struct EnvScope {
-  const bool outer = t_no_switches;
-  EnvScope() {
-    bool any = false;
-    for (char** e = environ; e && *e && !any; ++e) any = (*e)[0] == 'I' && strncmp(*e, "IFQ_", 4) == 0;
-    t_no_switches = !any;
-  }
-  ~EnvScope() { t_no_switches = outer; }
-};
-
+// A switch of the environment (getenv alone: a walk over `environ` would not be covered where the C library makes getenv
+// safe beside a setenv of another thread).  About 0.1 us a look, so the plans ask after their cheap conditions.
 int env_int(const char* name, int dflt) {
-  if (t_no_switches) return dflt;
   const char* v = getenv(name);
   return (v && *v) ? atoi(v) : dflt;
 }
@@ -463,10 +448,10 @@ cudaError_t launch_narrow(int cin, int pool, int cout, dim3 grid, dim3 block, co
 // at most 256 anchors, and the resident filters plus two staging and two band buffers within the
 // shared memory of one CTA.  Fills every field but the pointers.
 bool win_plan(const ifq_conv_desc* d, const ConvGeom& g, int nsm, WinArgs* wa, size_t* smem) {
-  if (env_int("IFQ_WIN", 1) == 0) return false;
   if (g.in8 || g.kb != 2) return false;
   const int k = d->kh;
   if (d->stride != 1 || d->kw != k || (k & 1) == 0 || k > 7 || 2 * d->pad != k - 1) return false;
+  if (env_int("IFQ_WIN", 1) == 0) return false;
   if (!(d->cin == 16 || d->cin % 32 == 0)) return false;
   int ct;
   if (d->cout == 32 || d->cout == 64) ct = d->cout;
@@ -567,12 +552,12 @@ bool win_wins(const ifq_conv_desc* d, const ConvGeom& g) {
 // a band of at least two output rows within the shared memory of one CTA.  Fills every field but
 // the pointers; *E and *NT select the instance.
 bool warp_plan(const ifq_conv_desc* d, const ConvGeom& g, WarpConvArgs* wa, size_t* smem, int* E, int* NT) {
-  if (env_int("IFQ_WARP", 1) == 0) return false;
   if (d->kh != 3 || d->kw != 3 || d->stride != 1 || d->pad != 1) return false;
   if (g.in8 ? d->cin != 4 : !(g.sbi == 2 && (d->cin == 8 || d->cin == 16))) return false;
   if (g.kb != 2 || !(d->cout == 8 || d->cout == 16 || d->cout == 32)) return false;
   if (g.pool != 1 && g.pool != 2) return false;
   if (g.pool == 2 && ((g.ho & 1) || (g.wo & 1))) return false;
+  if (env_int("IFQ_WARP", 1) == 0) return false;
   const int e = g.in8 ? 8 : d->cin, nt = d->cout / 8;
   const int pp = e / 8, ksd = (3 * pp + 3) / 4, nb = nt * 3 * ksd;
   const int strips = ceil_div(g.wo, 16);
@@ -1085,7 +1070,6 @@ double tc_cycles(const ConvGeom& g, int cout, int nsm, int bn, int ks, int gb, b
 // stack after the first), so the tensor-core kernel may load them before its dependency wait.
 int run_conv(const ifq_conv_desc* d, const void* x, const void* w_prep, const int32_t* thr, const int8_t* sign,
              void* y_codes, int32_t* y_acc, cudaStream_t st, bool early = false) {
-  const EnvScope env;
   ConvGeom g;
   int rc = check_conv(d, &g);
   if (rc) return rc;

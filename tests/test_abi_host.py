@@ -2,6 +2,8 @@
 against the oracle fold, synchronous argument errors, shapes and packed sizes."""
 import ctypes
 import re
+import shutil
+import subprocess
 
 import numpy as np
 import pytest
@@ -383,3 +385,15 @@ def test_prepared_filters_depend_on_the_filters_alone(cin, cout, k, kbits):
                             assert want in (None, got), (n, h, w, stride, pad, kb, pool, mode, path)
                             want = got
     assert want >= cout * K
+
+
+def test_switches_are_read_through_getenv_alone():
+    """The library never walks the environment itself: `environ` may move while another thread sets a variable, and a C
+    library can only guard its own getenv against that."""
+    nm = shutil.which("nm")
+    if nm is None:
+        pytest.skip("no nm")
+    ifq.lib()
+    names = subprocess.run([nm, "-D", "--undefined-only", ifq.lib_path()], capture_output=True, text=True, check=True).stdout
+    used = {ln.split()[-1].split("@")[0] for ln in names.splitlines() if ln.strip()}
+    assert "getenv" in used and not used & {"environ", "__environ", "_environ"}
