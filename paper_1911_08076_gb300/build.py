@@ -42,9 +42,9 @@ def _stale() -> bool:
     return any(os.path.getmtime(s) > t for s in _sources())
 
 
-# The warp-specialised tensor-core kernels run at the 72-register cap of 864 threads per CTA; every
-# instance must fit it without spilling to local memory (a build with spills is refused).
-_GUARDED = ("conv_tc_kernel", "conv_stack_kernel")
+# The warp-specialised tensor-core kernels run at the register cap of their CTA (72 registers at 864 threads, 80
+# at 768); every instance must fit it without spilling to local memory (a build with spills is refused).
+_GUARDED = ("conv_tc_kernel", "conv_stack_kernel", "conv_band_kernel", "conv_win_kernel")
 
 
 def spilling_kernels(ptxas_log: str):

@@ -46,8 +46,18 @@
 // shift-add to pack, where a compare per threshold takes six or more (k = 2) or a search (k = 3, 4).
 // Each column's line is fitted and then checked at every T_i and T_i + 1 with those same operations
 // when the CTA starts; between these the result cannot change because g is monotone in x and so is its
-// rounding.  Columns whose check fails (thresholds that are not equally spaced) make their block of 64
-// columns compare, as the im2col kernel's epilogue does.
+// rounding.  A block of 64 columns with a column whose check fails takes one of two slower forms:
+//   * 3- and 4-bit codes whose thresholds are nearly equally spaced (the separated conversion's, floored one by one):
+//     a line half a step lower is the code or one below it, and one comparison with the threshold that it names
+//     decides;
+//   * any others: three comparisons (2-bit codes) or a search of four steps.
+// Measured (us; im2col kernel, then here by line, line and comparison, search): 4-bit codes 3x3 384 -> 384 on 14 x 14 x
+// 256 images 64.7, 53.4, 60.7, 71.3, 1x1 128 -> 256 on 28 x 28 x 256 93.8, 26.8, 40.9, 62.9; 2-bit codes (line, three
+// comparisons) 38.6, 33.3, 37.9 and 37.9, 23.5, 32.8.  A 4-ary search by compares and selects took 78.0 and 79.1 where
+// the search takes 71.3 and 62.9, and spilled.  The form is one for all of a warp's channel tiles, in a loop of its own:
+// chosen unit by unit the network of 16 small layers took 1 % longer.
+// Every comparison is a saturating fma, sat(s A - T), of integers.  All instances fit 80 registers without spilling:
+// with the comparisons beside the lines' 32 registers they spilled (and a spill may move around a tensor-memory load).
 //
 // Measured (us; im2col kernel, this one): 3x3 256 -> 256 on 56 x 56 x 256 images 300, 167 (5.7 PTOPS; 59 % of the
 // instruction's rate); 1x1 512 -> 512 on 28 x 28 x 256 94.7, 43.3; 5x5 96 -> 256 on 27 x 27 x 128 43.5, 25.0; 3x3 1024
@@ -143,10 +153,32 @@ __device__ __forceinline__ void band_ld(uint32_t t0, uint32_t (&v)[16]) {
       : "memory");
 }
 
+// The same with 16 columns (k = 0, 1).
+__device__ __forceinline__ void band_ld16(uint32_t t0, uint32_t (&v)[8]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.16x256b.x2.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];\n\t"
+      "tcgen05.wait::ld.sync.aligned;"
+      : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7])
+      : "r"(t0)
+      : "memory");
+}
+
 // 8 packed bytes (32 two-bit fields) -> one slot: nibble i of register 2j holds field 16j + 2i, of
 // register 2j + 1 field 16j + 2i + 1.
 __device__ __forceinline__ uint4 band_expand(uint32_t w0, uint32_t w1) {
   return make_uint4(w0 & 0x33333333u, (w0 >> 2) & 0x33333333u, w1 & 0x33333333u, (w1 >> 2) & 0x33333333u);
+}
+
+// Shared memory at a 32-bit address that a code is part of (tables that do not change after the fit).
+__device__ __forceinline__ float lds_f(uint32_t addr) {
+  float v;
+  asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(addr));
+  return v;
+}
+__device__ __forceinline__ float4 lds_f4(uint32_t addr) {
+  float4 v;
+  asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr));
+  return v;
 }
 
 // The code of D against the column's line (a, b), as the low bits of the result: 2^23 + round(L sat(a D + b)).
@@ -168,13 +200,16 @@ __device__ __forceinline__ void band_code2(float d0, float d1, float2 l0, float2
 
 // Fits the line of one column: thresholds thr[0..L-1], sign s, |accumulator| <= B (LMAX: 3 or 15, the most that L
 // is).  Thresholds at or past the bound (never or always exceeded, as the conversion's saturated ones of a channel
-// with a small batch-norm scale) only have to stay past it.  Returns whether the line gives the exact code of
+// with a small batch-norm scale) only have to stay past it.  Returns kBandLine where the line gives the exact code of
 // every accumulator: with ascending thresholds it does when its code is at most i at x = T_i and at least i + 1
-// at x = T_i + 1 (i = 0..L-1, both within the bound), because it cannot decrease with x = s A.
+// at x = T_i + 1 (i = 0..L-1, both within the bound), because it cannot decrease with x = s A.  Else, for
+// LMAX = 15, the line half a step lower: kBandNear where that is the code or one below it (at most i at T_i, at least
+// i at T_i + 1), so that one comparison is left.  Else kBandFar.
 // LMAX = 15: the four lanes of a quad share a column, q-th lane thresholds i = q, q + 4, .. against all (105 pairs
 // in one thread took 5 us at the start of every launch).
+constexpr uint32_t kBandLine = 0, kBandNear = 1, kBandFar = 2;
 template <int LMAX>
-__device__ __forceinline__ bool band_fit(const int32_t* thr, int L, int s, int B, int q, float2* line) {
+__device__ __forceinline__ uint32_t band_fit(const int32_t* thr, int L, int s, int B, int q, float2* line) {
   constexpr int NQ = LMAX == 3 ? 1 : 4, NI = (LMAX + NQ - 1) / NQ;
   constexpr float kBig = 3.0e37f;
   const float fb = (float)B, fl = (float)L;
@@ -229,32 +264,83 @@ __device__ __forceinline__ bool band_fit(const int32_t* thr, int L, int s, int B
   const float m1 = 0.5f * (quad(mlo, true) + quad(mhi, false));
   // g(x) = (x - m1) / w + 1/2, x = s A = 2 s D;  v = g / L
   const float iw = 1.0f / (w * fl), fs = (float)s;
-  const float la = inside ? 2.0f * fs * iw : 0.0f, lb = inside ? 0.5f / fl - m1 * iw : (float)below / fl;
-  *line = make_float2(la, lb);
+  const float la = inside ? 2.0f * fs * iw : copysignf(0.0f, fs);   // (the sign is read from it: band_near)
+  float lb = inside ? 0.5f / fl - m1 * iw : (float)below / fl;
+  // the code at T_i at most i, at T_i + 1 at least i + up
+  auto check = [&](uint32_t up) {
+    bool good = ok;
 #pragma unroll
-  for (int k = 0; k < NI; ++k) {
-    const int i = NQ * k + q;
-    const uint32_t c0 = band_code(0.5f * fs * ti[k], la, lb, fl) & 0xFFu;
-    const uint32_t c1 = band_code(0.5f * fs * (ti[k] + 1.0f), la, lb, fl) & 0xFFu;
-    if (i < L) ok = ok && (ti[k] < -fb || c0 <= (uint32_t)i) && (ti[k] >= fb || c1 >= (uint32_t)(i + 1));
+    for (int k = 0; k < NI; ++k) {
+      const int i = NQ * k + q;
+      const uint32_t c0 = band_code(0.5f * fs * ti[k], la, lb, fl) & 0xFFu;
+      const uint32_t c1 = band_code(0.5f * fs * (ti[k] + 1.0f), la, lb, fl) & 0xFFu;
+      if (i < L) good = good && (ti[k] < -fb || c0 <= (uint32_t)i) && (ti[k] >= fb || c1 >= (uint32_t)i + up);
+    }
+    if constexpr (NQ == 4) {   // all four lanes'
+      const uint32_t votes = __ballot_sync(0xffffffffu, good);
+      good = (votes >> (threadIdx.x & 28) & 15u) == 15u;
+    }
+    return good;
+  };
+  uint32_t kind = check(1u) ? kBandLine : kBandFar;
+  if constexpr (LMAX == 15) {
+    if (kind != kBandLine && inside) lb = -m1 * iw;
+    if (check(0u) && kind != kBandLine) kind = kBandNear;
   }
-  return ok;
+  *line = make_float2(la, lb);
+  return kind;
 }
 
-// The code of D against a column's own thresholds (where no line separates them), as band_code's result:
-// t = (-T1, -T2, -T3, 2 s) and three saturating fmas, or up to 15 ascending ones as a 4-ary search over
-// {T3, T7, T11, 2 s}, {T0, T1, T2, -}, {T4, ..}, ..
+// Codes where some column of a block has no line, as band_code's results, two rows (D0, D1) of a column at a time.
+// They are sums of saturating fmas, sat(2 s D - T) = [s A > T] (every T is an integer), added in pairs.
+__device__ __forceinline__ uint64_t band_pair(float a, float b) {
+  uint64_t r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ uint64_t band_add2(uint64_t a, uint64_t b) {
+  uint64_t r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ void band_split(uint64_t v, uint32_t& a, uint32_t& b) {
+  asm("mov.b64 {%0, %1}, %2;" : "=r"(a), "=r"(b) : "l"(v));
+}
+// A column's thresholds in shared memory: (-T0, -T1, -T2, 2 s) for 2-bit codes, else sixteen -T in a row (-inf past the
+// last), then 2 s.
+__host__ __device__ constexpr int band_thr_bytes(int sbo) { return sbo == 2 ? 16 : 80; }
+
+// `t`: the column's table.  4-bit codes are searched for in four steps, each one threshold.
 template <int SBO>
-__device__ __forceinline__ uint32_t band_code_cmp(float d, const float4* t) {
-  const float4 h = t[0];
+__device__ __forceinline__ void band_codes_far(float d0, float d1, uint32_t t, uint32_t& c0, uint32_t& c1) {
+  uint64_t n = band_pair(kBandMagic, kBandMagic);
   if constexpr (SBO == 2) {
-    return __float_as_uint(kBandMagic + (sat_fma(d, h.w, h.x) + sat_fma(d, h.w, h.y) + sat_fma(d, h.w, h.z)));
+    const float4 h = lds_f4(t);
+    n = band_add2(n, band_pair(sat_fma(d0, h.w, h.x), sat_fma(d1, h.w, h.x)));
+    n = band_add2(n, band_pair(sat_fma(d0, h.w, h.y), sat_fma(d1, h.w, h.y)));
+    n = band_add2(n, band_pair(sat_fma(d0, h.w, h.z), sat_fma(d1, h.w, h.z)));
+    band_split(n, c0, c1);
   } else {
-    const float x = d * h.w;
-    const uint32_t q = (uint32_t)(x > h.x) + (uint32_t)(x > h.y) + (uint32_t)(x > h.z);
-    const float4 g = t[1 + q];
-    return 0x4B000000u + 4u * q + (uint32_t)(x > g.x) + (uint32_t)(x > g.y) + (uint32_t)(x > g.z);
+    const float s2 = lds_f(t + 64u), m = lds_f(t + 28u);
+    c0 = __float_as_uint(fmaf(sat_fma(d0, s2, m), 8.0f, kBandMagic));
+    c1 = __float_as_uint(fmaf(sat_fma(d1, s2, m), 8.0f, kBandMagic));
+#pragma unroll
+    for (int k = 4; k >= 1; k >>= 1) {   // [s A > T_(c + k - 1)]
+      const uint32_t tk = t + 4u * (uint32_t)(k - 1) - 4u * 0x4B000000u;
+      c0 = __float_as_uint(fmaf(sat_fma(d0, s2, lds_f(tk + 4u * c0)), (float)k, __uint_as_float(c0)));
+      c1 = __float_as_uint(fmaf(sat_fma(d1, s2, lds_f(tk + 4u * c1)), (float)k, __uint_as_float(c1)));
+    }
   }
+}
+
+// From a line that is the code c or one below it: c + [s A > T_c].  (With an exact line s A <= T_c.)
+__device__ __forceinline__ void band_codes_near(float d0, float d1, float2 line, uint64_t fl2, uint32_t t, uint32_t& c0,
+                                                uint32_t& c1) {
+  band_code2(d0, d1, line, line, fl2, c0, c1);
+  const float t0 = lds_f(t + 4u * c0 - 4u * 0x4B000000u), t1 = lds_f(t + 4u * c1 - 4u * 0x4B000000u);
+  const float s2 = copysignf(2.0f, line.x);
+  band_split(band_add2(band_pair(__uint_as_float(c0), __uint_as_float(c1)),
+                       band_pair(sat_fma(d0, s2, t0), sat_fma(d1, s2, t1))), c0, c1);
 }
 
 // Position in a ring of n buffers and the parity of its pass.
@@ -563,8 +649,8 @@ __global__ void __launch_bounds__(kBandThreads, 1)
   uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw_ + 127) & ~(uintptr_t)127);
   const uint32_t sbase = smem_u32(smem);
   float2* sLin = (float2*)(smem + a.off_lin);        // [ngrp * BN] (a, b)
-  float4* sThr = (float4*)(smem + a.off_thr);        // their thresholds (band_code_cmp)
-  uint32_t* sBad = (uint32_t*)(smem + a.off_bad);    // per warp of the fit: some line failed its check
+  float4* sThr = (float4*)(smem + a.off_thr);        // their thresholds (band_codes_far)
+  uint32_t* sBad = (uint32_t*)(smem + a.off_bad);    // per warp of the fit: the worst kind of its columns
   uint32_t* sTab = (uint32_t*)(smem + a.off_tab);    // A descriptors of the MMAs of a chunk
   uint32_t* tmem_slot = (uint32_t*)(smem + a.off_bad + 128);
   const uint32_t bar = sbase + a.off_bar;
@@ -738,18 +824,18 @@ __global__ void __launch_bounds__(kBandThreads, 1)
       const int32_t* T = a.thr + (size_t)(has ? nn : 0) * a.lvl;
       const int s = has ? a.sign[nn] : 1, L = has ? a.lvl : 0;
       float2 ln;
-      const bool good = band_fit<SBO == 2 ? 3 : 15>(T, L, s, a.bound, q, &ln);
+      const uint32_t kind = band_fit<SBO == 2 ? 3 : 15>(T, L, s, a.bound, q, &ln);
       if (q == 0) sLin[c] = has ? ln : make_float2(0.f, 0.f);
       auto th = [&](int i) { return i < L ? (float)T[i] : INFINITY; };
       if constexpr (SBO == 2) {
         sThr[c] = make_float4(-th(0), -th(1), -th(2), 2.0f * (float)s);
       } else {
-        sThr[5 * c + 1 + q] = make_float4(th(4 * q), th(4 * q + 1), th(4 * q + 2), 0.f);
-        if (q == 0) sThr[5 * c] = make_float4(th(3), th(7), th(11), 2.0f * (float)s);
+        sThr[5 * c + q] = make_float4(-th(4 * q), -th(4 * q + 1), -th(4 * q + 2), -th(4 * q + 3));
+        if (q == 0) sThr[5 * c + 4].x = 2.0f * (float)s;
       }
-      // a bit per column, or four of them (any: the block of 64 columns compares)
-      const bool bad = __any_sync(0xffffffffu, has && !good);
-      if (lane == 0) sBad[c4 >> 5] = bad ? 1u : 0u;
+      // the worst of a warp's columns
+      const uint32_t worst = __reduce_max_sync(0xffffffffu, has ? kind : kBandLine);
+      if (lane == 0) sBad[c4 >> 5] = worst;
     }
     named_bar(1, 32 * kEW);
     bool ok = true;
@@ -759,46 +845,32 @@ __global__ void __launch_bounds__(kBandThreads, 1)
     BandRing ar, fr;                                  // the unit's accumulator and its barriers
     ar.add(eg, a.nacc);
     fr.add(eg, a.ncb);
-    int jt = eg / per_tile, rest = eg - jt * per_tile;   // its tile, its place in the tile
-    int cur_t = -1, cur_f = -1, pixel = -1;
-    bool bad = false;
-    float2 line[NC];                                  // this thread's columns: 8 k + 2 quad, + 1
-#pragma unroll 1
-    for (; jt < n_local; ar.add(EG, a.nacc), fr.add(EG, a.ncb)) {
-      const int t = rest / a.mt, m = rest - t * a.mt;
-      if (t != cur_t) {                               // the channel tile's lines stay in registers
-        cur_t = t;
-        const float4* l4 = (const float4*)(sLin + t * BN + cblk + 2 * quad);
-#pragma unroll
-        for (int k = 0; k < NC / 2; ++k) {
-          const float4 l = l4[4 * k];
-          line[2 * k] = make_float2(l.x, l.y);
-          line[2 * k + 1] = make_float2(l.z, l.w);
-        }
-        bad = false;                                  // some column of the block
-#pragma unroll
-        for (int i = 0; i < 2 * NQ; ++i) bad = bad || sBad[((t * BN + cblk) * NQ >> 5) + i] != 0;
-      }
+    int rest = eg % per_tile;                         // its place in the tile
+    int tile = first + eg / per_tile * step;
+    const int msh = a.mt >> 1;                        // (one or two subtiles)
+    // One unit of channel tile t in the given form; line: with kBandLine, this thread's columns 8 k +
+    // 2 quad, + 1 (the other forms read what they need, so that no register holds a line there).  False after a
+    // timeout.
+    auto unit = [&](auto kind_c, const int t, const float2* line) __attribute__((always_inline)) {
+      constexpr uint32_t kind = decltype(kind_c)::value;
+      const int m = rest & (a.mt - 1);
       // the output pixel of row `lane` of the quarter, -1 for an anchor that is none
-      const int f0 = ((first + jt * step) * a.mt + m) * 128 + quarter * 32;
-      if (f0 != cur_f) {
-        cur_f = f0;
-        const int f = f0 + lane;
-        const int rr = fdiv31(f, a.div_P), xx = f - rr * a.P;
-        const int b = fdiv31(rr, a.div_HP), yy = rr - b * a.HP;
-        pixel = b < a.n && yy < a.oh && xx < a.ow ? (b * a.oh + yy) * a.ow + xx : -1;
-      }
-      ok = __all_sync(0xffffffffu, mbar_wait_backoff(c_full(fr.i), fr.ph, 32));
+      const int f = (tile * a.mt + m) * 128 + quarter * 32 + lane;
+      const int rr = fdiv31(f, a.div_P), xx = f - rr * a.P;
+      const int b = fdiv31(rr, a.div_HP), yy = rr - b * a.HP;
+      const int pixel = b < a.n && yy < a.oh && xx < a.ow ? (b * a.oh + yy) * a.ow + xx : -1;
+      if (!__all_sync(0xffffffffu, mbar_wait_backoff(c_full(fr.i), fr.ph, 32))) return false;
       const uint32_t tacc = tmem + (uint32_t)(ar.i * BN + cblk) + ((uint32_t)(quarter * 32 + 16 * half0) << 16);
-      if (!ok) break;
       tc_fence_after();
       const int ch0 = (nt0 + t) * BN + cblk + NC * quad;   // this thread's first output channel
       const bool chans = ch0 < a.cout;
 #pragma unroll 1
       for (int h = 0; h < NH; ++h) {
         uint32_t packed[2][kW];                       // rows lane / 4 and lane / 4 + 8 of the half
-        const int lr = 16 * (half0 + h) + (lane >> 2);
-        const int pix0 = __shfl_sync(0xffffffffu, pixel, lr), pix1 = __shfl_sync(0xffffffffu, pixel, lr + 8);
+        // the output pixel of row r (asked for where it is used: two registers fewer)
+        auto pix_of = [&](int r) {
+          return __shfl_sync(0xffffffffu, pixel, 16 * (half0 + h) + 8 * r + (lane >> 2));
+        };
         const uint32_t lo16 = (uint32_t)(16 * h) << 16;
 #pragma unroll
         for (int r = 0; r < 2; ++r)
@@ -807,9 +879,9 @@ __global__ void __launch_bounds__(kBandThreads, 1)
 #pragma unroll
         for (int ld = NL - 1; ld >= 0; --ld) {        // descending, so that the first code ends up lowest
           uint32_t v[16];
-          band_ld(tacc + lo16 + (uint32_t)(32 * ld), v);
-          if (a.y_codes) {
-            if (!bad) {
+          if constexpr (kind == kBandLine) {
+            band_ld(tacc + lo16 + (uint32_t)(32 * ld), v);
+            if (a.y_codes) {
 #pragma unroll
               for (int r = 0; r < 2; ++r)
 #pragma unroll
@@ -821,27 +893,36 @@ __global__ void __launch_bounds__(kBandThreads, 1)
                   w = (w << SBO) + c1;
                   w = (w << SBO) + c0;
                 }
-            } else {
-              // thresholds that no line separates: compared
-              constexpr int kT = SBO == 2 ? 1 : 5;
-              const float4* th = sThr + (size_t)(t * BN + cblk + 32 * ld + 2 * quad) * kT;
+            }
+          } else {
+            // thresholds that no line separates: 16 columns at a time, in a loop (the registers of more spill)
+#pragma unroll 1
+            for (int g = 1; g >= 0; --g) {
+              const int c16 = 32 * ld + 16 * g;
+              uint32_t u[8];
+              band_ld16(tacc + lo16 + (uint32_t)c16, u);
 #pragma unroll
-              for (int j = 7; j >= 0; --j) {
-                const float4* tj = th + (8 * (j >> 1) + (j & 1)) * kT;
-#pragma unroll
-                for (int r = 0; r < 2; ++r) {
-                  uint32_t& w = packed[r][(8 * ld + j) * SBO / 32];
-                  w = (w << SBO) + band_code_cmp<SBO>(__uint_as_float(v[4 * (j >> 1) + 2 * r + (j & 1)]), tj);
-                }
+              for (int j = 3; j >= 0; --j) {          // channel 8 ld + 4 g + j
+                const float d0 = __uint_as_float(u[4 * (j >> 1) + (j & 1)]), d1 = __uint_as_float(u[4 * (j >> 1) + 2 + (j & 1)]);
+                const int col = t * BN + cblk + c16 + 2 * quad + 8 * (j >> 1) + (j & 1);
+                const uint32_t tab = sbase + a.off_thr + (uint32_t)(col * band_thr_bytes(SBO));
+                uint32_t c0, c1;
+                if constexpr (kind == kBandNear) band_codes_near(d0, d1, sLin[col], fl2, tab, c0, c1);
+                else band_codes_far<SBO>(d0, d1, tab, c0, c1);
+                uint32_t& w0 = packed[0][8 * ld * SBO / 32];
+                uint32_t& w1 = packed[1][8 * ld * SBO / 32];
+                w0 = (w0 << SBO) + c0;
+                w1 = (w1 << SBO) + c1;
               }
             }
           }
           if (a.y_acc) {
+            if constexpr (kind != kBandLine) band_ld(tacc + lo16 + (uint32_t)(32 * ld), v);
             // A = 2 D as an integer: the low mantissa bits of 2 D + 1.5 * 2^23
             auto ia = [&](int i) { return __float_as_int(fmaf(__uint_as_float(v[i]), 2.0f, 12582912.0f)) - 0x4B400000; };
 #pragma unroll
             for (int r = 0; r < 2; ++r) {
-              const int pix = r ? pix1 : pix0;
+              const int pix = pix_of(r);
               if (pix < 0) continue;
               int32_t* dst = a.y_acc + (size_t)pix * a.cout + ch0 + 8 * ld;
               if ((a.cout & 3) == 0) {
@@ -858,11 +939,12 @@ __global__ void __launch_bounds__(kBandThreads, 1)
             }
           }
         }
-        if (a.y_codes && chans) {
+        if (a.y_codes) {
+          const int pix0 = pix_of(0), pix1 = pix_of(1);
           // what the exponent bits of the terms add up to (0x4B000000 each, shifted)
           constexpr uint32_t kOff = SBO == 2 ? 0xE7000000u : 0xFB000000u;
 #pragma unroll
-          for (int r = 0; r < 2; ++r) {
+          for (int r = 0; r < 2 && chans; ++r) {
             const int pix = r ? pix1 : pix0;
             if (pix < 0) continue;
             uint8_t* dst = a.y_codes + (size_t)pix * rowb + ((ch0 * SBO) >> 3);
@@ -886,8 +968,41 @@ __global__ void __launch_bounds__(kBandThreads, 1)
       rest += EG;
       while (rest >= per_tile) {
         rest -= per_tile;
-        ++jt;
+        tile += step;
       }
+      ar.add(EG, a.nacc);
+      fr.add(EG, a.ncb);
+      return true;
+    };
+    // this warp's blocks (one a channel tile) all take the form that the worst of them needs
+    uint32_t kind = kBandLine;
+#pragma unroll 1
+    for (int t = 0; t < ntl; ++t)
+#pragma unroll
+      for (int i = 0; i < 2 * NQ; ++i) kind = max(kind, sBad[((t * BN + cblk) * NQ >> 5) + i]);
+    if (kind == kBandLine) {
+#pragma unroll 1
+      while (ok && tile < a.mtiles) {
+        const int t = rest >> msh;
+        float2 line[NC];                              // a channel tile's lines stay in registers
+        const float4* l4 = (const float4*)(sLin + t * BN + cblk + 2 * quad);
+#pragma unroll
+        for (int k = 0; k < NC / 2; ++k) {
+          const float4 l = l4[4 * k];
+          line[2 * k] = make_float2(l.x, l.y);
+          line[2 * k + 1] = make_float2(l.z, l.w);
+        }
+#pragma unroll 1
+        do {
+          ok = unit(std::integral_constant<uint32_t, kBandLine>{}, t, line);
+        } while (ok && tile < a.mtiles && rest >> msh == t);
+      }
+    } else if (SBO == 4 && kind == kBandNear) {
+#pragma unroll 1
+      while (ok && tile < a.mtiles) ok = unit(std::integral_constant<uint32_t, kBandNear>{}, rest >> msh, nullptr);
+    } else {
+#pragma unroll 1
+      while (ok && tile < a.mtiles) ok = unit(std::integral_constant<uint32_t, kBandFar>{}, rest >> msh, nullptr);
     }
   }
 

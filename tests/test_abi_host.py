@@ -246,6 +246,15 @@ ptxas info    : Compiling entry function '_ZN3ifq14conv_tc_kernelILi64ELi16ELi2E
     assert B.spilling_kernels("") == []
 
 
+@pytest.mark.parametrize("kernel", ["16conv_band_kernelILi128ELi4EE", "15conv_win_kernelILi1ELi0EE"])
+def test_build_refuses_spills_of_every_tcgen05_kernel(kernel):
+    from paper_1911_08076_gb300 import build as B
+    log = f"""ptxas info    : Compiling entry function '_ZN3ifq{kernel}Ev' for 'sm_103a'
+    8 bytes stack frame, 4 bytes spill stores, 12 bytes spill loads
+"""
+    assert B.spilling_kernels(log) == [f"_ZN3ifq{kernel}Ev"]
+
+
 def test_graph_with_copies_validates_the_stack_before_any_capture():
     """ifq_graph_create_io checks the stack (and a missing output handle) on the host first, like
     ifq_graph_create (works without a GPU)."""

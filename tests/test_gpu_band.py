@@ -1,7 +1,7 @@
 """The band kernel (4-bit products on an input band expanded once) on every launch shape of its table, bit-exact
 against the CPU oracle: ragged maps and channel tiles, each load granule (16, 8, 4, 2 and 1 bytes), odd plane
 counts, several chunks and tiles, strided 1 x 1 filters, 2-, 3- and 4-bit codes, and thresholds that saturate or are not
-equally spaced (compared one by one instead of by the fitted line).  The results are integers: no tolerance."""
+equally spaced (one comparison after the fitted line, or a search).  The results are integers: no tolerance."""
 import numpy as np
 import pytest
 import torch
@@ -32,14 +32,19 @@ CASES = [
 ]
 
 
-def _thresholds(rng, cout, K, kbits, even):
-    """Ascending thresholds across the accumulator's spread: floors of equally spaced values, or any."""
+def _thresholds(rng, cout, K, kbits, spacing):
+    """Ascending thresholds across the accumulator's spread: floors of equally spaced values ("even"), some of them a
+    fraction of a step off ("near", as the separated conversion's), or any ("far").  By the kernel's fit a line is the
+    code, the code or one below it, or neither; the last two only in some columns of a block."""
     L = (1 << kbits) - 1
     sd = np.sqrt(K * L * (2 * L + 1) / 6.0)
     step, base = rng.uniform(0.3, 1.0, cout) * 3 * sd / L, rng.normal(0, 0.3 * sd, cout)
     step[1::5] *= 10.0 ** rng.integers(-1, 5, step[1::5].shape)   # steep ones, and thresholds past the bound L K
     T = np.floor(base[:, None] + step[:, None] * (np.arange(L) - (L - 1) / 2))
-    if not even:
+    if spacing == "near":
+        T[::4] += np.floor(rng.uniform(-0.2, 0.2, T[::4].shape) * step[::4, None])
+        T.sort(axis=1)
+    elif spacing == "far":
         T[::3] += np.cumsum(rng.integers(0, int(sd) + 2, T[::3].shape), axis=1)
     return np.clip(T, -L * K - 1, L * K).astype(np.int32), np.where(rng.integers(0, 4, cout) == 0, -1, 1).astype(np.int8)
 
@@ -56,8 +61,8 @@ def test_every_launch_shape_matches_oracle(case, monkeypatch):
     prep = torch.empty(ifq.ifq_weights_prep_bytes(d), dtype=torch.uint8, device="cuda")
     ifq.ifq_pack_weights(d, torch.from_numpy(synth.pack_signs(wt).view(np.int32)).cuda(), prep)
     rowb = cout * synth.field_bits(kbits) // 8
-    for even in (True, False):
-        T, s = _thresholds(rng, cout, k * k * cin, kbits, even)
+    for spacing in ("even", "near", "far"):
+        T, s = _thresholds(rng, cout, k * k * cin, kbits, spacing)
         C = O.int_chain(A, T, s)
         for shape in range(1, 2 + SHAPES):   # 1: the planner's choice
             monkeypatch.setenv("IFQ_BAND", str(shape))
@@ -66,7 +71,7 @@ def test_every_launch_shape_matches_oracle(case, monkeypatch):
             ifq.ifq_conv2bit(d, xp, prep, torch.from_numpy(T).cuda(), torch.from_numpy(s).cuda(), yc, ya)
             assert ifq.ifq_device_status() == ifq.IFQ_OK
             assert (ya.cpu().numpy() == A).all(), shape
-            assert (synth.unpack_codes(yc.cpu().numpy(), cout, kbits) == C).all(), (shape, even)
+            assert (synth.unpack_codes(yc.cpu().numpy(), cout, kbits) == C).all(), (shape, spacing)
 
 
 @pytest.mark.parametrize("kbits,K", [(2, 65536), (3, 28064), (4, 13088)])
