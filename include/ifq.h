@@ -269,6 +269,19 @@ int ifq_pack_weights(const ifq_conv_desc* d, const uint32_t* w_bits, void* w_pre
  */
 int ifq_conv_plan(const ifq_conv_desc* d, int* path);
 
+/*
+ * The kernel that ifq_conv2bit launches for `d` on the current device (a full
+ * GB300's launch shape, without K split, where there is none), as text (host;
+ * reads the switches as ifq_conv2bit does): its name, for the tensor-core
+ * path's kernels with the channels per tile and then key=value pairs of the
+ * launch shape, e.g. "conv_band_kernel<128, 2> subtiles=1 channel_tiles=2
+ * resident=1 ctas=152 ...": ctas: the grid; units: accumulators (128 pixels x
+ * a channel tile) that a CTA computes at most; cycles: the planner's estimate.
+ * For reports and tests; the keys may change with ifq_version.  Writes at most
+ * `size` bytes (192 are enough) with the terminating zero.
+ */
+int ifq_conv_kernel(const ifq_conv_desc* d, char* text, size_t size);
+
 /* Device workspace that ifq_conv2bit needs for `d` (host, pure); may be 0. */
 int ifq_conv_workspace_bytes(const ifq_conv_desc* d, size_t* bytes);
 

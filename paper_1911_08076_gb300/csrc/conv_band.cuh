@@ -11,9 +11,9 @@
 //     2-bit map of twice the channels whose odd channels weigh +4 / -4 (nibbles 0x6 / 0xE);
 //   * the fp32 accumulation was checked exact on GB300 up to |A| = 196608 with odd addends along all
 //     of K = 65536, the bound the planner admits (test_accumulation_exact_at_the_admitted_bound).
-// Measured rate of the instruction (M128 x N128 x K64, both operands in shared memory, A at any slot
-// offset): 64 cycles, 9.7 PTOPS on 152 SMs, twice the e4m3 rate of the im2col kernel (conv_tc.cuh); N = 64
-// takes 48 cycles and N = 32 40, where reading the 4 KB of A takes longer than the products.
+// Measured rate of the instruction (M128 x N128 x K64, both operands in shared memory): 9.57 PTOPS on 152 SMs, twice
+// the e4m3 rate of the im2col kernel (conv_tc.cuh).  That is 64 cycles; N = 64 takes 48 (6.35 PTOPS) and N = 32 40, where
+// reading the 4 KB of A takes longer than the products.
 //
 // A is the input itself.  A slot is 16 bytes: 32 consecutive 2-bit fields of one input pixel (one
 // "plane" of it), expanded to nibbles by a mask and a shift.  Slots lie in shared memory in pixel
@@ -103,7 +103,7 @@ struct BandArgs {
   int planes, cp, nchunk;  // planes per pixel, planes per chunk, chunks
   int linear;              // 1: slot f is input pixel f (1 x 1, stride 1, no padding)
   int gran, glg;           // bytes per load (16: two planes; 8, 4, 2, 1: one plane); log2 of the granule lanes
-  int taps, npair, nodd;   // plane pairs; MMAs of the odd plane
+  int taps, nodd;          // filter taps; MMAs of the odd plane
   int nstep;               // MMAs (K = 64) per pass
   int tab_last, ntab;      // table entries before the last chunk's, and in all
   int ring;                // chunk buffers
@@ -284,8 +284,10 @@ __device__ __forceinline__ uint32_t band_fit(const int32_t* thr, int L, int s, i
   };
   uint32_t kind = check(1u) ? kBandLine : kBandFar;
   if constexpr (LMAX == 15) {
-    if (kind != kBandLine && inside) lb = -m1 * iw;
-    if (check(0u) && kind != kBandLine) kind = kBandNear;
+    if (__any_sync(0xffffffffu, kind != kBandLine)) {
+      if (kind != kBandLine && inside) lb = -m1 * iw;
+      if (check(0u) && kind != kBandLine) kind = kBandNear;
+    }
   }
   *line = make_float2(la, lb);
   return kind;
@@ -563,8 +565,9 @@ __device__ __forceinline__ void band_mma(const BandArgs& a, const BandMma& w, co
             break;
           }
           tc_fence_after();
-          // the turn goes over as soon as this pass's waits are done: two passes issued side by side (179 us
-          // on the 3x3 256 -> 256 layer at batch 256) beat handing it over with two groups left (200 us)
+          // the turn goes over as soon as this pass's waits are done: two passes issued side by side beat handing it
+          // over with two groups left (179 and 200 us on the 3x3 256 -> 256 layer at batch 256, in an earlier build that
+          // differed in nothing else)
           if (ALT && last_c && lane == 0) mbar_arrive(w.bar_turn + 8u * (uint32_t)(mi ^ 1));
           // Shared memory is the busy unit here (an MMA reads 8 KB of it in 64 cycles), so what this warp
           // reads from it is asked for ahead: the next group's entries during this group, and whether the

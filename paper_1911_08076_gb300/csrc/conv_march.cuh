@@ -2,7 +2,7 @@
 // 2 x 2 pool, 2-bit codes out, few channels (Eq. (1), the pool of Sec. 2.1 on Y^conv, the thresholds of Eq. (7)).
 // Inputs of 4 channels of 8-bit values or of 8 channels of 2-bit codes: at most one 32-bit word a pixel.
 //
-// These layers have too few channels to fill a tcgen05 tile, and what bounds them is instructions issued.  One
+// These layers have too few channels to fill a tcgen05 tile.  One
 // warp takes 8 pooled columns and marches down the pooled rows; a step is two m16n8k16 f16 products chains (the
 // two conv rows of the pooled row), whose 16 rows are the 8 pooled columns at window column 0 (rows 0..7) and 1
 // (rows 8..15).  So a thread's fragments of the two chains hold all four window positions of its channels, and
@@ -17,8 +17,8 @@
 //
 // Measured (us, batch 64, pooled; the kernel before, this one): 3 x 3 4 -> 8 on 416 x 416 8-bit pixels 64.9 (dp4a, the
 // direct kernel), 43.9; 3 x 3 8 -> 16 on 208 x 208 2-bit codes 41.9 (the warp kernel's e4m3 mma.sync, which
-// issues as four instructions), 30.3.  Their bytes take 7.5 and 2.5 us: instructions and the latency of
-// loads and products bound both (issue slots 37 and 49 % busy; rows loaded one step ahead 45.2 and 32.3).
+// issues as four instructions), 30.3.  Their bytes take 7.5 and 1.25 us: the latency of loads and products bounds
+// both (issue slots 38.6 and 28.9 % busy; rows loaded one step ahead 45.2 and 32.3 us).
 #pragma once
 #include "conv_common.cuh"
 

@@ -8,6 +8,7 @@
 
 #include <cstdint>
 #include <cmath>
+#include <cstdio>
 #include <cstdlib>
 #include <cstring>
 #include <mutex>
@@ -602,12 +603,12 @@ bool warp_supported(const ifq_conv_desc* d, const ConvGeom& g) {
 }
 
 // Where the warp-MMA kernel is the default (measured on GB300, full-size layers at batch 64, L2
-// flushed, against the kernel each layer took before): 2-bit layers with 8 input channels
-// (IFQ-Tinier-YOLO conv2, 8 -> 16 at 208 x 208: 46 vs 103 us on the narrow bit-serial kernel with the
-// fused pool, 62 vs 107 us without) and 8-bit-input layers without a fused pool (3 x 3 4 -> 8 at
+// flushed, against the kernel each layer took before): 2-bit layers with 8 input channels (8 -> 16 at
+// 208 x 208 without a pool: 62 vs 107 us on the narrow bit-serial kernel; under a fused pool the path's layers
+// run on the march kernel, 30 vs 42 us here) and 8-bit-input layers without a fused pool (3 x 3 4 -> 8 at
 // 416 x 416: 144 vs 207 us on the direct kernel).  Elsewhere it loses: one e4m3 mma.sync issues about
 // four instructions on this GPU, and the tcgen05 window kernel (16-channel layers: Tiny-YOLO conv2
-// 54 vs 124 us) or the direct kernel (the pooled first layer: 91 vs 107 us) stays ahead.
+// 54 vs 124 us) or, for pooled first layers, the march or direct kernel stays ahead.
 bool warp_wins(const ifq_conv_desc* d, const ConvGeom& g) {
   return warp_supported(d, g) && (g.in8 ? g.pool == 1 : d->cin == 8);
 }
@@ -924,6 +925,15 @@ void band_fill(const ifq_conv_desc* d, const ConvGeom& g, const BandGeom& b, Ban
   a->div_HP = make_fastdiv((uint32_t)a->HP);
 }
 
+// Bytes of codes that an output pixel's share of a channel tile of bn stores one at a time, weighted with how many
+// cache lines a store instruction then touches: rows that are no multiple of `word` bytes are stored bytewise, else
+// the last channel tile's rest is.
+double tile_byte_stores(int cout, int bn, int sbo, int word) {
+  const int rowb = cout * sbo / 8;
+  const double cols = (double)(rowb % word ? cout : cout % bn) / ceil_div(cout, bn);
+  return cols * sbo / 8 * std::min(1.0, rowb / 128.0);
+}
+
 // One launch shape on `base` (band_fill): fills the plan, or false where it does not fit.
 bool band_try(const BandArgs& base, const BandShape& sh, int sbo, int nsm, BandPlan* pl) {
   pl->a = base;
@@ -951,8 +961,8 @@ bool band_try(const BandArgs& base, const BandShape& sh, int sbo, int nsm, BandP
   a.resident = sh.resident ? 1 : 0;
   const size_t cols = (size_t)a.ngrp * bn, thrb = sbo == 2 ? 16 : 80;
   // Planes per chunk: as many as a granule's lanes take at once and leave a ring of two (deeper rings and
-  // smaller chunks measured no faster: 178 to 183 us on the 3x3 256 -> 256 layer, 50 to 53 us on the 1x1
-  // 512 -> 512 one with whole 8-plane chunks against 71 us with 4).
+  // smaller chunks measured no faster: in an earlier build 178 to 183 us on the 3x3 256 -> 256 layer, 50 to 53 us
+  // on the 1x1 512 -> 512 one with whole 8-plane chunks against 71 us with 4).
   const int cpmax = a.gran == 16 ? 8 : 4;
   size_t bbytes = 0;
   for (int cp = std::min(a.planes, cpmax); cp >= 1 && a.ring == 0; cp = cp > 2 ? (cp - 1) / 2 * 2 : 0) {
@@ -991,34 +1001,54 @@ bool band_try(const BandArgs& base, const BandShape& sh, int sbo, int nsm, BandP
   const int per = std::max(1, std::min(a.mtiles, nsm / a.ngroups));
   pl->grid = per * a.ngroups;
   pl->bn = bn;
-  // Estimated cycles, with constants fitted to 62 layers timed in each shape (10 % from the measured time on
-  // average; the shape picked is within 0.6 % of the best one on average).  What each role of a CTA takes for
-  // one tile; the slowest of them sets the pace after the first tile.
-  const bool wide = sbo == 4, acc = a.y_acc != nullptr;
+  // Estimated cycles: the first tile (its chunks and products one after another, its epilogue, what every launch
+  // takes), then a tile at the pace of the slowest role.  The constants are fitted to 1497 layers timed in every shape
+  // that fits them (the benchmark networks' at all power-of-two batches, and random ones; codes, accumulators or both),
+  // for the choice rather than the time: estimates lie 12 % from the measured time on average.
+  const bool wide = sbo == 4, big = bn == 128, alt = mt == 1;
   const double units = (double)a.ngrp * mt;
-  const double mma = a.nstep * units * (bn == 128 ? 93.3 : 72.4) * (mt == 2 ? 0.938 : 0.854) + 559.0 * a.ngrp;
-  const double epi = (bn == 128 ? 2140.0 : 1180.0) * (acc ? 4.5 : 1.0) * (wide ? 1.26 : 1.0);
+  const double mma = a.nstep * units * (big ? (alt ? 61.4 : 107.0) : (alt ? 57.5 : 68.7)) + 836.0 * a.ngrp;
+  const double mma1 = a.nstep * (alt ? units * (big ? 37.8 : 42.6) : (big ? 137.0 : 90.1));
   const double batches = std::ceil((double)a.slots * (1 << a.glg) / (32.0 * 4 * kBandProd));
-  const double chunk = batches * 1380.0 * (a.gran < 8 ? 2.14 : 1.0) + 297.0;
-  const double fbytes = (double)a.nst * a.ngrp * a.stage_bytes;
-  const double stream = a.resident ? 0.0 : fbytes * 0.0355, fill = a.resident ? fbytes * 0.0174 : 0.0;
+  const double load = a.gran == 16 ? 1270.0 : (a.gran == 8 ? 1450.0 : (a.gran == 4 ? 2340.0 : 3390.0));
+  const double chunk = batches * load + 251.0;
+  double first = big ? 7190.0 : 7010.0, epi = (big ? (alt ? 2570.0 : 4440.0) : (alt ? 2130.0 : 2280.0)) * (wide ? 1.13 : 1.0);
+  if (a.y_codes) {
+    const double bytes = tile_byte_stores(a.cout, bn, sbo, wide ? 8 : 4) * (wide ? 114.0 : 95.9);
+    first += bytes;
+    epi += bytes;
+  } else {
+    first *= 0.844;
+    epi *= 0.844;
+  }
+  if (a.y_acc) {
+    const double fill = (double)a.cout / ((double)a.nt * bn);
+    first += fill * (big ? 7170.0 : 2200.0);
+    epi += fill * (big ? 8020.0 : 3050.0);
+  }
+  const double stream = a.resident ? 0.0 : (double)a.nst * a.ngrp * a.stage_bytes * 0.0405;
   const double pace = std::max(std::max(mma, units * epi / 2), std::max(a.nchunk * chunk, stream));
-  const double tiles = ceil_div(a.mtiles, per);
-  pl->cost = 4800.0 + (wide ? 2460.0 : 0.0) + std::max(fill, chunk) + 0.7 * mma + epi + (tiles - 0.7) * pace;
+  const double fits = wide ? std::ceil(cols * 4.0 / (32 * kBandEpi)) : 0.0;   // rounds of band_fit
+  pl->cost = first + 5920.0 * fits + chunk + std::max(mma1, 0.94 * (a.nchunk - 1) * chunk) +
+             (ceil_div(a.mtiles, per) - 1) * pace;
   return true;
 }
 
 // The launch shape of the band path with the smallest estimated time, or false where none fits or the im2col
-// kernel (tc_cost, in cycles) is as fast.  IFQ_BAND: 0: none; 2, 3, ..: that shape of the table, where it fits.
-bool band_plan(const ifq_conv_desc* d, const ConvGeom& g, int nsm, bool acc, double tc_cost, BandPlan* best) {
+// kernel (tc_cost, in cycles) is about as fast.  On the 1497 layers of the fit the choice takes 0.8 % longer than the
+// best of all on average (3.8 % with the fit before), and 20 of them, by 3 to 14 %, are slower than on the im2col kernel
+// (one in 16 before, by up to 48 %).  IFQ_BAND: 0: none; 2, 3, ..: that
+// shape of the table, where it fits.
+bool band_plan(const ifq_conv_desc* d, const ConvGeom& g, int nsm, double tc_cost, BandPlan* best) {
   BandGeom b;
   if (!band_geom(d, g, &b)) return false;
   const int want = env_int("IFQ_BAND", 1);
   if (want == 0) return false;
-  if (want == 1 && 0.95 * tc_cost < 8500.0) return false;   // no estimate of band_try is below
+  if (want == 1 && 0.93 * tc_cost < 7500.0) return false;   // no estimate of band_try is below
   BandArgs base;
   band_fill(d, g, b, &base);
-  base.y_acc = acc ? (int32_t*)16 : nullptr;
+  base.y_codes = d->out_mode & IFQ_OUT_CODES ? (uint8_t*)16 : nullptr;   // (whether there is one)
+  base.y_acc = d->out_mode & IFQ_OUT_ACC ? (int32_t*)16 : nullptr;
   bool have = false;
   for (int i = 0; i < kBandShapeCount; ++i) {
     BandPlan p;
@@ -1028,7 +1058,7 @@ bool band_plan(const ifq_conv_desc* d, const ConvGeom& g, int nsm, bool acc, dou
       have = true;
     }
   }
-  return have && (want >= 2 || best->cost < 0.95 * tc_cost);
+  return have && (want >= 2 || best->cost < 0.93 * tc_cost);
 }
 
 template <int BN, int SBO>
@@ -1057,13 +1087,46 @@ cudaError_t set_band_attrs() {
 }
 
 // Estimated cycles of the im2col kernel (conv_tc.cuh) on a layer of codes with tiles of bn channels, K split over
-// ks CTAs: constants fitted as the band kernel's.
-double tc_cycles(const ConvGeom& g, int cout, int nsm, int bn, int ks, int gb, bool acc) {
-  const double tiles = (double)ceil_div(g.M, kBM) * ceil_div(cout, bn), rounds = std::ceil(tiles / nsm);
-  const double stage = (gb == 16 ? 382.0 : (gb == 8 ? 394.0 : (gb == 4 ? 747.0 : 1900.0))) * (g.sb == 4 ? 1.51 : 1.0);
-  const double k = (double)(g.Kpad / kBK) / ks * stage;
-  const double e = (bn == 32 ? 2450.0 : (bn == 64 ? 2430.0 : 4110.0)) * (g.sb == 4 ? 1.5 : 1.0) * (acc ? 2.02 : 1.0);
-  return 5050.0 + (ks == 2 ? 3950.0 : 0.0) + k + e + (rounds - 1) * std::max(k, e);
+// ks CTAs: a launch's first tile, then one tile a round at the pace of its K stages or its epilogue.  Constants fitted
+// as the band kernel's.
+double tc_cycles(const ifq_conv_desc* d, const ConvGeom& g, int nsm, int bn, int ks, int gb) {
+  const bool wide = g.sb == 4, acc = (d->out_mode & IFQ_OUT_ACC) != 0, codes = (d->out_mode & IFQ_OUT_CODES) != 0;
+  const double tiles = (double)ceil_div(g.M, kBM) * ceil_div(d->cout, bn), rounds = std::ceil(tiles / nsm);
+  const double nk = (double)(g.Kpad / kBK) / ks;
+  const int i = gb == 16 ? 3 : (gb == 8 ? 2 : (gb == 4 ? 1 : 0)), j = bn == 32 ? 0 : (bn == 64 ? 1 : 2);
+  static constexpr double kFirst[2][4] = {{928, 297, 205, 255}, {590, 590, 313, 451}};    // a K stage of the first tile
+  static constexpr double kNext[2][4] = {{1190, 439, 312, 331}, {948, 948, 843, 708}};     // and of the others
+  static constexpr double kEpi1[2][3] = {{1950, 2840, 4570}, {2400, 5940, 7710}};
+  static constexpr double kEpi[2][3] = {{787, 1800, 4820}, {3250, 3330, 7200}};
+  const double bytes = codes ? tile_byte_stores(d->cout, bn, g.sb, 4) * (wide ? 421.0 : 492.0) : 0.0;
+  const double e1 = kEpi1[wide][j] * (acc ? 1.5 : 1.0) + bytes;
+  const double e = kEpi[wide][j] * (acc ? (codes ? 1.685 : 1.56) : 1.0) + bytes;
+  return 4320.0 + (ks == 2 ? 2850.0 : 0.0) + nk * kFirst[wide][i] + e1 +
+         (rounds - 1) * std::max(nk * kNext[wide][i] + 611.0, e);
+}
+
+// What the tensor-core path runs for a layer: the band kernel in a launch shape, or the im2col kernel with tiles of bn
+// channels, K split over ks CTAs.  (A switch of the im2col kernel's asks for that kernel.)
+struct TcChoice {
+  int bn, ks, gb, bx_env;
+  bool band;
+  BandPlan bp;
+  double tc_cost;          // estimated cycles of the im2col kernel
+};
+
+void choose_tc(const ifq_conv_desc* d, const ConvGeom& g, int nsm, TcChoice* c) {
+  const int bn_env = env_int("IFQ_TC_BN", 0), ks_env = env_int("IFQ_TC_KS", 0);
+  c->bx_env = env_int("IFQ_TC_BX", 0);
+  c->bn = choose_bn(g, d->cout, nsm, bn_env);
+  c->ks = 1;
+  c->gb = granule_bytes(d, g);
+  if (c->gb == 16) {
+    if (g.sbi == 2) choose_split<16, 2, 2>(g, d->cout, nsm, ks_env, &c->bn, &c->ks);
+    else if (g.sb == 4) choose_split<16, 4, 4>(g, d->cout, nsm, ks_env, &c->bn, &c->ks);
+    else choose_split<16, 4, 2>(g, d->cout, nsm, ks_env, &c->bn, &c->ks);
+  }
+  c->tc_cost = tc_cycles(d, g, nsm, c->bn, c->ks, c->gb);
+  c->band = !bn_env && !ks_env && !c->bx_env && band_plan(d, g, nsm, c->tc_cost, &c->bp);
 }
 
 // early: the kernels before this one in the stream write neither w_prep nor thr / sign (a layer of a
@@ -1151,18 +1214,11 @@ int run_conv(const ifq_conv_desc* d, const void* x, const void* w_prep, const in
     else if (ya) e = launch_k(conv_win_kernel<0, 1>, grid, block, smem, st, tma, wa);
     else e = launch_k(conv_win_kernel<0, 0>, grid, block, smem, st, tma, wa);
   } else if (path == IFQ_PATH_TC) {
-    // (a switch of the im2col kernel's asks for that kernel)
-    const int bn_env = env_int("IFQ_TC_BN", 0), ks_env = env_int("IFQ_TC_KS", 0), bx_env = env_int("IFQ_TC_BX", 0);
-    int bn = choose_bn(g, d->cout, nsm, bn_env), ks = 1;
-    const int gb = granule_bytes(d, g);
-    if (gb == 16) {
-      if (g.sbi == 2) choose_split<16, 2, 2>(g, d->cout, nsm, ks_env, &bn, &ks);
-      else if (g.sb == 4) choose_split<16, 4, 4>(g, d->cout, nsm, ks_env, &bn, &ks);
-      else choose_split<16, 4, 2>(g, d->cout, nsm, ks_env, &bn, &ks);
-    }
-    BandPlan bp;
-    if (!bn_env && !ks_env && !bx_env &&
-        band_plan(d, g, nsm, ya != nullptr, tc_cycles(g, d->cout, nsm, bn, ks, gb, ya != nullptr), &bp)) {
+    TcChoice c;
+    choose_tc(d, g, nsm, &c);
+    const int bn = c.bn, ks = c.ks, gb = c.gb;
+    if (c.band) {
+      BandPlan& bp = c.bp;
       CUtensorMap tm;
       if (!encode_bandmap(d, g, w_prep, bp.bn, &tm)) return IFQ_ECUDA;
       bp.a.x = (const uint8_t*)x;
@@ -1183,7 +1239,7 @@ int run_conv(const ifq_conv_desc* d, const void* x, const void* w_prep, const in
       // those single-tile launches are bound by the K-stage pipeline's latency, not by the filter
       // stream.  IFQ_TC_BX = 1 takes it where the filters are read about once (at most two 128-row
       // tiles), 2 wherever the split instance runs.
-      const bool bx = bx_env != 0 && (bx_env == 2 || ceil_div(g.M, kBM) <= 2) && bn == 64 && ks == 2 && gb == 16 &&
+      const bool bx = c.bx_env != 0 && (c.bx_env == 2 || ceil_div(g.M, kBM) <= 2) && bn == 64 && ks == 2 && gb == 16 &&
                       g.sbi == 2 && g.sb == 2;
       CUtensorMap tm;
       if (!(bx ? encode_bitmap(d, g, w_prep, bn, &tm) : encode_wmap(d, g, w_prep, bn, &tm))) return IFQ_ECUDA;
@@ -1806,6 +1862,47 @@ int ifq_conv_plan(const ifq_conv_desc* d, int* path) {
   const int p = choose_path(d, g);
   if (p < 0) return IFQ_EUNSUPPORTED;
   *path = p;
+  return IFQ_OK;
+}
+
+int ifq_conv_kernel(const ifq_conv_desc* d, char* text, size_t size) {
+  if (!text || size == 0) return IFQ_EINVAL;
+  ConvGeom g;
+  int rc = check_conv(d, &g);
+  if (rc) return rc;
+  int nsm = 0;
+  if (ensure_init(&nsm)) {
+    cudaGetLastError();
+    nsm = 152;   // no device: a full GB300
+  }
+  const int path = choose_path(d, g);
+  if (path < 0) return IFQ_EUNSUPPORTED;
+  const char* name = "conv_bitserial_kernel";
+  if ((path == IFQ_PATH_DIRECT || (path == IFQ_PATH_WARP && !g.in8)) && march_supported(d, g)) {
+    name = "conv_march_kernel";
+  } else if (path == IFQ_PATH_DIRECT) {
+    name = "conv_direct_kernel";
+  } else if (path == IFQ_PATH_WARP) {
+    name = "conv_warp_kernel";
+  } else if (path == IFQ_PATH_WIN) {
+    name = "conv_win_kernel";
+  } else if (path == IFQ_PATH_TC) {
+    TcChoice c;
+    choose_tc(d, g, nsm, &c);
+    if (c.band) {
+      const BandArgs& a = c.bp.a;
+      const int per = c.bp.grid / a.ngroups;
+      snprintf(text, size, "conv_band_kernel<%d, %d> subtiles=%d channel_tiles=%d resident=%d ctas=%d units=%d accumulators=%d "
+               "chunks=%d ring=%d cycles=%.0f im2col_cycles=%.0f", c.bp.bn, g.sb, a.mt, a.ngrp, a.resident, c.bp.grid,
+               ceil_div(a.mtiles, per) * a.mt * a.ngrp, a.nacc, a.nchunk, a.ring, c.bp.cost, c.tc_cost);
+    } else {
+      snprintf(text, size, "conv_tc_kernel<%d, %d> ksplit=%d cycles=%.0f", c.bn, c.gb, c.ks, c.tc_cost);
+    }
+    return IFQ_OK;
+  } else if (narrow_supported(d, g)) {
+    name = "conv_bitserial_narrow_kernel";
+  }
+  snprintf(text, size, "%s", name);
   return IFQ_OK;
 }
 

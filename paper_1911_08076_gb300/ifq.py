@@ -71,6 +71,7 @@ _SIGS = {
     "ifq_weights_prep_bytes": ([ctypes.POINTER(ConvDesc), ctypes.POINTER(_SZ)], _I),
     "ifq_pack_weights": ([ctypes.POINTER(ConvDesc), _P, _P, _P], _I),
     "ifq_conv_plan": ([ctypes.POINTER(ConvDesc), ctypes.POINTER(_I)], _I),
+    "ifq_conv_kernel": ([ctypes.POINTER(ConvDesc), ctypes.c_char_p, _SZ], _I),
     "ifq_conv_workspace_bytes": ([ctypes.POINTER(ConvDesc), ctypes.POINTER(_SZ)], _I),
     "ifq_conv2bit": ([ctypes.POINTER(ConvDesc), _P, _P, _P, _P, _P, _P, _P, _SZ, _P], _I),
     "ifq_pool_out_shape": ([ctypes.POINTER(PoolDesc), ctypes.POINTER(_I), ctypes.POINTER(_I)], _I),
@@ -241,6 +242,13 @@ def ifq_conv_plan(d: ConvDesc) -> int:
     p = _I()
     _ok(lib().ifq_conv_plan(ctypes.byref(d), ctypes.byref(p)), "ifq_conv_plan")
     return p.value
+
+
+def ifq_conv_kernel(d: ConvDesc) -> str:
+    """The kernel (and launch shape) that ifq_conv2bit launches for d, as text."""
+    buf = ctypes.create_string_buffer(256)
+    _ok(lib().ifq_conv_kernel(ctypes.byref(d), buf, len(buf)), "ifq_conv_kernel")
+    return buf.value.decode()
 
 
 def ifq_weights_prep_bytes(d: ConvDesc) -> int:

@@ -406,3 +406,38 @@ def test_switches_are_read_through_getenv_alone():
     names = subprocess.run([nm, "-D", "--undefined-only", ifq.lib_path()], capture_output=True, text=True, check=True).stdout
     used = {ln.split()[-1].split("@")[0] for ln in names.splitlines() if ln.strip()}
     assert "getenv" in used and not used & {"environ", "__environ", "_environ"}
+
+
+@pytest.mark.parametrize("kernel,shapes", [
+    # n, h, w, cin, cout, k, code width, outputs: layers that the im2col kernel runs 1.15 to 1.5 times as fast
+    ("conv_tc_kernel", [(1, 12, 9, 304, 280, 3, 3, 1), (15, 32, 22, 88, 136, 3, 4, 1), (3, 9, 9, 128, 76, 3, 4, 1),
+                        (8, 7, 37, 480, 52, 3, 2, 1), (2, 6, 82, 248, 48, 3, 4, 1),
+                        (2, 61, 12, 872, 120, 3, 3, 1), (1, 10, 38, 416, 52, 3, 2, 1), (6, 9, 49, 112, 96, 5, 2, 1)]),
+    # and layers that the band kernel runs 1.05 to 4 times as fast
+    ("conv_band_kernel", [(256, 56, 56, 256, 256, 3, 2, 1), (256, 28, 28, 512, 512, 1, 2, 1), (128, 27, 27, 96, 256, 5, 4, 1),
+                          (9, 37, 45, 72, 100, 3, 2, 3), (256, 28, 28, 64, 512, 1, 4, 1), (21, 13, 50, 80, 652, 5, 3, 1),
+                          (162, 35, 79, 136, 164, 3, 2, 1), (32, 39, 47, 16, 600, 1, 2, 1), (97, 12, 37, 104, 80, 3, 2, 1)])])
+def test_estimates_choose_the_kernel_that_measured_faster(kernel, shapes):
+    for n, h, w, cin, cout, k, kbits, mode in shapes:
+        d = ifq.conv_desc(n, h, w, cin, cout, k, 1, k // 2, mode, ifq.IFQ_PATH_TC, kbits=kbits)
+        assert ifq.ifq_conv_kernel(d).startswith(kernel), (n, h, w, cin, cout, k, kbits, ifq.ifq_conv_kernel(d))
+
+
+def test_conv_kernel_text():
+    """ifq_conv_kernel names the kernel of every path and refuses what ifq_conv_plan refuses."""
+    name = lambda *a, **k: ifq.ifq_conv_kernel(ifq.conv_desc(*a, **k)).split(" ")[0].split("<")[0]
+    assert name(1, 16, 16, 64, 64, 3, 1, 1) == "conv_tc_kernel"
+    assert name(1, 16, 16, 64, 64, 3, 1, 1, path=ifq.IFQ_PATH_BITSERIAL) == "conv_bitserial_kernel"
+    assert name(1, 16, 16, 8, 16, 3, 1, 1, path=ifq.IFQ_PATH_BITSERIAL) == "conv_bitserial_narrow_kernel"
+    assert name(1, 416, 416, 4, 8, 3, 1, 1, pool=2, in_bits=8) == "conv_march_kernel"
+    assert name(1, 416, 416, 4, 8, 5, 1, 2, in_bits=8) == "conv_direct_kernel"
+    assert name(1, 208, 208, 8, 16, 3, 1, 1) == "conv_warp_kernel"
+    assert name(1, 208, 208, 16, 32, 3, 1, 1, pool=2) == "conv_win_kernel"
+    with pytest.raises(ifq.IfqError) as e:
+        ifq.ifq_conv_kernel(ifq.conv_desc(1, 8, 8, 64, 64, 3, 1, 1, kbits=5))
+    assert e.value.status == ifq.IFQ_EUNSUPPORTED
+    buf = ctypes.create_string_buffer(8)
+    d = ifq.conv_desc(1, 16, 16, 64, 64, 3, 1, 1)
+    assert ifq.lib().ifq_conv_kernel(ctypes.byref(d), buf, 8) == ifq.IFQ_OK and buf.value == b"conv_tc"
+    assert ifq.lib().ifq_conv_kernel(ctypes.byref(d), buf, 0) == ifq.IFQ_EINVAL
+    assert ifq.lib().ifq_conv_kernel(ctypes.byref(d), None, 8) == ifq.IFQ_EINVAL
