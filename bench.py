@@ -4,12 +4,12 @@
 A step is one pass of a layer stack over one batch through ifq_forward, replayed
 as a CUDA graph.  The headline workload is the largest single-GPU configuration:
 the 3x3 256->256 binary x 2-bit conv at 56x56, batch 256 (GEMM M = 802816,
-N = 256, K = 2304, 947 GOP).  The same JSON line carries a sub-record for every
+N = 256, K = 2304, 947 GOP).  The same JSON line carries a small record for every
 other configuration (the single PR1 layer, the ResNet-18 body b32, AlexNet
 conv2-FC7 b128, Tiny-YOLO and Tinier-YOLO b64 with fused pools, IFQ-Tinier-YOLO
-end to end from 8-bit pixels, the 1x1 512->512 layer b256), each with its step
-time, TOPS, images/s, roofline fraction, per-layer times, end-to-end figure and
-the oracle's CPU baseline.
+end to end from 8-bit pixels, the 1x1 512->512 layer b256): step time, TOPS,
+images/s, roofline fraction and end-to-end figure.  Their per-layer times, timing
+notes and the oracle's CPU baselines go to _build/bench_detail.json.
 
 Inputs are seeded synthetic codes already resident in HBM; L2 is flushed (a
 256 MB write) between timed steps, outside the per-step CUDA events.  `e2e`
@@ -60,6 +60,7 @@ PROFILES = os.path.join(ROOT, "profiles")
 KERNEL_DIR = os.path.join(ROOT, "paper_1911_08076_gb300", "csrc")
 RATES_SRC = os.path.join(ROOT, "bench_rates.cu")
 RATES_LIB = os.path.join(ROOT, "_build", "libbench_rates.so")
+DETAIL = os.path.join(ROOT, "_build", "bench_detail.json")
 
 
 def log(*a):
@@ -237,6 +238,42 @@ class ClockSampler:
                 "samples": len(sm)}
 
 
+MAX_LINE = 3500             # bytes of the printed line: what reads it may keep only the end of the output
+
+
+def brief(rec, keys):
+    """The given keys of a record, floats to five significant digits."""
+    r5 = lambda v: float(f"{v:.5g}") if isinstance(v, float) else v
+    return {k: r5(rec[k]) for k in keys if rec.get(k) is not None}
+
+
+def short_line(line, detail):
+    """The printed JSON line: the headline's figures in full, one small record for each other workload.  Per-layer
+    times, timing notes and everything else are in the file `detail`."""
+    out = {k: v for k, v in line.items() if k not in ("roofline", "e2e", "int8_peak", "rates_measured", "cpu_baseline",
+                                                      "layers_timed_alone", "configs", "pool_hbm")}
+    r = line["roofline"]
+    out["roofline"] = brief(r, ("bound", "achieved", "peak", "unit", "frac", "traffic", "kernel", "peak_source",
+                                "algorithmic_bytes_per_launch", "avg_launch_us"))
+    out["e2e"] = brief(line["e2e"], ("value", "unit", "h2d_bytes_per_step", "d2h_bytes_per_step", "ms_per_step"))
+    out["rates_tops"] = brief(line["rates_measured"], sorted(k for k in line["rates_measured"] if k.endswith("_tops")))
+    if line.get("cpu_baseline"):
+        out["cpu_baseline"] = brief(line["cpu_baseline"], ("value", "unit", "cores", "kind"))
+    out["pool_hbm"] = brief(line["pool_hbm"], ("us", "achieved_gbs", "frac"))
+    out["configs"] = {}
+    for name, rec in line["configs"].items():
+        c = brief(rec, ("ms_per_step", "value", "images_per_s", "gpu_launches"))
+        c["frac"] = brief(rec["roofline"], ("frac",)).get("frac")
+        c["e2e"] = brief(rec["e2e"], ("value", "h2d_bytes_per_step", "d2h_bytes_per_step"))
+        out["configs"][name] = c
+    out["detail"] = detail
+    text = json.dumps(out)
+    if len(text) > MAX_LINE:      # the headline alone rather than a line that is cut
+        out["configs"] = f"in {detail}"
+        text = json.dumps(out)
+    return text
+
+
 def line_config(wl, args):
     """The `config` object of both arms' JSON lines (identical for the same workload)."""
     convs = [l for l in wl.layers if l.kind == "conv"]
@@ -389,21 +426,11 @@ def job_throughput(ops_per_rank_step: float, world: int, step_ms_max: float) -> 
     return world * ops_per_rank_step / (step_ms_max * 1e-3) / 1e12
 
 
-PATH_NAMES = {0: "auto", 1: "conv_band_kernel or conv_tc_kernel", 2: "bitserial",
-              3: "conv_direct_kernel or conv_march_kernel", 4: "conv_win_kernel",
-              5: "conv_warp_kernel or conv_march_kernel"}
-
-
 def kernel_of(ifq, st, li):
-    """Name of the kernel family a layer launches (the planner's choice for convs)."""
+    """Name of the kernel a layer launches (the planner's choice for convs, with its tile)."""
     rec = st.layers[li]
     if rec.kind == ifq.IFQ_LAYER_CONV:
-        p = ifq.ifq_conv_plan(rec.conv)
-        if p == ifq.IFQ_PATH_BITSERIAL:
-            l = st.wl.layers[li]
-            narrow = l.kind == "conv" and l.cin in (4, 8, 16) and l.k == 3 and l.stride == 1 and l.cout <= 32
-            return "conv_bitserial_narrow_kernel" if narrow else "conv_bitserial_kernel"
-        return PATH_NAMES.get(p, str(p))
+        return re.sub(r" \w+=.*", "", ifq.ifq_conv_kernel(rec.conv))
     if rec.kind == ifq.IFQ_LAYER_POOL:
         return "maxpool_codes"
     return "fixed_output_kernel"
@@ -657,7 +684,10 @@ def run_ours(args):
     line["configs"] = subs
     line["pool_hbm"] = measure_pool_hbm(ifq, torch, dev, stream)
     if rank == 0:
-        print(json.dumps(line), flush=True)
+        os.makedirs(os.path.dirname(DETAIL), exist_ok=True)
+        with open(DETAIL, "w") as f:
+            json.dump(line, f, indent=1)
+        print(short_line(line, os.path.relpath(DETAIL, ROOT)), flush=True)
     if world > 1:
         dist.destroy_process_group()
 

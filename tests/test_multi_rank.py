@@ -103,3 +103,38 @@ def test_bench_counts_the_resnet18_step_ops_and_algorithmic_bytes():
     assert abs(sum(bench.conv_ops(l, B) for l in convs) - ops) < 1
     assert abs(sum(bench.alg_bytes(l, B, 2) for l in convs) - nbytes) < 1
     assert round(ops / 1e9, 1) == 108.5 and round(nbytes / 1e6, 1) == 31.2
+
+
+def test_bench_prints_a_line_that_can_be_read_whole():
+    """The printed line stays short with every workload in it, whatever the names and notes of the full record, and
+    keeps the keys of the bench's contract."""
+    import json
+
+    import bench
+    rec = {"ms_per_step": 0.1234567891234, "value": 5381.223456789, "images_per_s": 1454545.4545454545, "gpu_launches": 20000,
+           "roofline": {"bound": "tensor", "achieved": 5400.123456789, "peak": 9700.123456789, "unit": "TFLOP/s",
+                        "frac": 0.5567891234, "traffic": 63223040.0, "kernel": "conv_band_kernel<128, 2>",
+                        "peak_source": "x" * 90, "algorithmic_bytes_per_launch": 102834176.123, "avg_launch_us": 174.123456,
+                        "timing": "y" * 400, "vs_measured_rates": {"note": "z" * 400}},
+           "e2e": {"value": 1415.123456789, "unit": "TOPS", "h2d_bytes_per_step": 51380224, "d2h_bytes_per_step": 51380224,
+                   "ms_per_step": 0.669123456789, "sequence": "s" * 300},
+           "layers_timed_alone": [{"name": "layer", "kernel": "k" * 60}] * 20,
+           "cpu_baseline": {"value": 0.0923456789, "unit": "TOPS", "cores": 16, "kind": "oracle", "sample": "t" * 300}}
+    args = type("A", (), {"gpus": 8, "path": "auto"})()
+    line = dict(rec, metric=bench.METRIC, unit=bench.UNIT, n_gpus=8, steps=200, warmup=20, higher_is_better=True, scaling="weak",
+                vs_baseline=None, dtype="d" * 80, data="synthetic",
+                config=bench.line_config(bench.synth.get(bench.HEADLINE), args), pct_of_int8_peak=3434.123456789,
+                int8_peak={"tops": 158.0, "source": "u" * 200}, timed_wall_s=0.0912345678,
+                rates_measured={f"rate_{i}_tops": 4784.123456789 for i in range(5)} | {"how": "v" * 300},
+                clocks={"sm_mhz": 2070.0, "sm_max_mhz": 2070.0, "reasons": [], "samples": 31},
+                pool_hbm={"us": 40.9123456, "achieved_gbs": 5396.123456, "frac": 0.80812345, "shape": "w" * 80},
+                configs={n: rec for n in bench.SUB_WORKLOADS})
+    text = bench.short_line(line, "_build/bench_detail.json")
+    got = json.loads(text)
+    assert "\n" not in text and len(text) <= bench.MAX_LINE and set(got["configs"]) == set(bench.SUB_WORKLOADS)
+    for k in ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling", "vs_baseline",
+              "dtype", "data", "config", "gpu_launches", "clocks"):
+        assert got[k] == line[k]
+    assert set(got["e2e"]) >= {"value", "unit", "h2d_bytes_per_step", "d2h_bytes_per_step"}
+    assert abs(got["e2e"]["value"] / rec["e2e"]["value"] - 1) < 1e-4
+    assert len(bench.short_line(dict(line, configs={f"n{i}": rec for i in range(40)}), "f")) <= bench.MAX_LINE
