@@ -15,10 +15,10 @@ Inputs are seeded synthetic codes already resident in HBM; L2 is flushed (a
 256 MB write) between timed steps, outside the per-step CUDA events.  `e2e`
 replays a graph from ifq_graph_create_io that also copies the pinned host input
 in and every result out, one launch per step.  `roofline` is the conv kernel
-against the tensor peak of e2m1 operands (the measured bf16 peak x 5: kind::mxf4
-K = 64 products over bf16), with the DRAM traffic of the committed ncu summary of the same workload and kernel source;
-beside it, fractions against the e4m3 tcgen05 and the s8 mma.sync rates
-measured in the same process.
+against the tensor rate of e2m1 operands (tcgen05 kind::mxf4, measured in the same
+process), with the DRAM traffic of the committed ncu summary of the same workload and
+kernel source; beside it, fractions against the e4m3 tcgen05 and the s8 mma.sync rates
+measured in the same process and the measured bf16 burst.
 
     python bench.py [--gpus N] [--steps K] [--warmup W] [--impl reference] [--workload NAME] [--no-sub]
 
@@ -54,7 +54,7 @@ UNIT = "TOPS"
 HEADLINE = "roofline3x3"
 SUB_WORKLOADS = ["pr1", "resnet18", "alexnet", "tinyyolo_fused", "tinieryolo_fused", "tinieryolo_full_fused",
                  "roofline1x1"]
-FP4_PER_BF16 = 5.0          # tcgen05.mma kind::mxf4 M128 N128 K64: 64 cycles, 9.7 PTOPS on 152 SMs, over 1.95 PFLOP/s bf16
+FP4_PER_BF16 = 5.0          # assumed mxf4 / bf16 ratio, where the rate probe cannot run
 FALLBACK_BF16_TFLOPS = 1900.0
 PROFILES = os.path.join(ROOT, "profiles")
 KERNEL_DIR = os.path.join(ROOT, "paper_1911_08076_gb300", "csrc")
@@ -157,8 +157,9 @@ def build_rates(force: bool = False) -> str:
 
 
 def measure_rates(stream):
-    """Tensor rates measured now, on this GPU: tcgen05 e4m3 at N = 128 and 256 (the conv's
-    instruction) and mma.sync s8 (the dense INT8 path)."""
+    """Tensor rates measured now, on this GPU: tcgen05 mxf4 at N = 32, 64 and 128 (the band kernel's
+    instruction), e4m3 at N = 128 and 256 (the im2col and window kernels') and mma.sync s8 (the
+    dense INT8 path)."""
     try:
         L = ctypes.CDLL(build_rates())
     except Exception as e:  # no nvcc or no library: report the reason, not a guess
@@ -167,6 +168,11 @@ def measure_rates(stream):
     L.bench_tc_e4m3_tops.argtypes = [ctypes.c_int, ctypes.c_int, ctypes.c_int, ctypes.c_void_p, ctypes.POINTER(dbl)]
     L.bench_mma_s8_tops.argtypes = [ctypes.c_int, ctypes.c_int, ctypes.c_void_p, ctypes.POINTER(dbl)]
     out = {}
+    L.bench_tc_mxf4_tops.argtypes = L.bench_tc_e4m3_tops.argtypes
+    for n in (32, 64, 128):
+        v = dbl(0.0)
+        rc = L.bench_tc_mxf4_tops(n, 8192, 5, ctypes.c_void_p(stream.cuda_stream), ctypes.byref(v))
+        out[f"tcgen05_mxf4_n{n}_tops"] = v.value if rc == 0 else None
     L.bench_tc_e4m3_tops_a.argtypes = [ctypes.c_int, ctypes.c_int, ctypes.c_int, ctypes.c_int, ctypes.c_void_p,
                                        ctypes.POINTER(dbl)]
     for n in (128, 256):
@@ -179,8 +185,9 @@ def measure_rates(stream):
     v = dbl(0.0)
     rc = L.bench_mma_s8_tops(4096, 3, ctypes.c_void_p(stream.cuda_stream), ctypes.byref(v))
     out["mma_sync_s8_tops"] = v.value if rc == 0 else None
-    out["how"] = ("same process, before the timed regions: one CTA per SM issuing M128xNxK32 e4m3 tcgen05 MMAs "
-                  "back to back (A in shared memory; tmem_a: A in tensor memory, as the conv issues them); "
+    out["how"] = ("same process, before the timed regions: one CTA per SM issuing M128xNxK64 mxf4 or M128xNxK32 e4m3 "
+                  "tcgen05 MMAs back to back (A in shared memory; tmem_a: A in tensor memory, as the im2col kernel "
+                  "issues them); "
                   "4 CTAs x 8 warps per SM issuing m16n8k32 s8 mma.sync; 2 ops per MAC")
     return out
 
@@ -629,9 +636,11 @@ def run_ours(args):
     stream = torch.cuda.Stream(device=dev)
     flush = torch.empty(256 << 20, dtype=torch.uint8, device=dev)
     bf16, bf16_sus, hbm, src = read_peaks()
-    peaks = {"tensor_tops": bf16 * FP4_PER_BF16, "hbm_gbs": hbm,
-             "tensor_source": f"{src} bf16 burst {bf16} x {FP4_PER_BF16} (kind::mxf4 K = 64 over bf16, measured)"}
     rates = measure_rates(stream)
+    mxf4 = rates.get("tcgen05_mxf4_n128_tops")
+    peaks = {"tensor_tops": mxf4 or bf16 * FP4_PER_BF16, "hbm_gbs": hbm,
+             "tensor_source": "tcgen05 kind::mxf4 M128 N128 K64 rate measured in this process" if mxf4 else
+                              f"{src} bf16 burst {bf16} x {FP4_PER_BF16} (assumed)"}
     K, W = args.steps, args.warmup
 
     head, wl, x, params = measure_workload(args.workload, args, ifq, torch, dev, stream, flush, K, W, world,
@@ -644,12 +653,13 @@ def run_ours(args):
         return ach / v if v else None
 
     r["vs_measured_rates"] = {
+        f"{src}_bf16_burst": frac(bf16),
+        "tcgen05_mxf4_n128": frac(rates.get("tcgen05_mxf4_n128_tops")),
         "tcgen05_e4m3_n128": frac(rates.get("tcgen05_e4m3_n128_tops")),
         "tcgen05_e4m3_n256": frac(rates.get("tcgen05_e4m3_n256_tops")),
         "tcgen05_e4m3_tmem_a_n128": frac(rates.get("tcgen05_e4m3_tmem_a_n128_tops")),
-        "note": "achieved / the e4m3 tcgen05 rate measured in this process (the im2col kernel's "
-                "instruction; the band kernel multiplies e2m1 at twice that rate; "
-                "tmem_a: with A in tensor memory, the operand form the conv issues)"}
+        "note": "achieved / the rates measured in this process (mxf4: the band kernel's instruction; e4m3: the im2col "
+                "and window kernels', tmem_a with A in tensor memory as the im2col kernel issues it) and the bf16 burst"}
     s8 = rates.get("mma_sync_s8_tops")
     line = {
         "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": K, "warmup": W,
