@@ -12,8 +12,8 @@
 //   * the fp32 accumulation was checked exact on GB300 up to |A| = 196608 with odd addends along all
 //     of K = 65536, the bound the planner admits (test_accumulation_exact_at_the_admitted_bound).
 // Measured rate of the instruction (M128 x N128 x K64, both operands in shared memory): 9.57 PTOPS on 152 SMs, twice
-// the e4m3 rate of the im2col kernel (conv_tc.cuh).  That is 64 cycles; N = 64 takes 48 (6.35 PTOPS) and N = 32 40, where
-// reading the 4 KB of A takes longer than the products.
+// the e4m3 rate of the im2col kernel (conv_tc.cuh).  That is 64 cycles; N = 64 takes 48 (6.31 PTOPS) and N = 32 46 (3.31),
+// where reading the 4 KB of A takes longer than the products.
 //
 // A is the input itself.  A slot is 16 bytes: 32 consecutive 2-bit fields of one input pixel (one
 // "plane" of it), expanded to nibbles by a mask and a shift.  Slots lie in shared memory in pixel
@@ -59,11 +59,11 @@
 // Every comparison is a saturating fma, sat(s A - T), of integers.  All instances fit 80 registers without spilling:
 // with the comparisons beside the lines' 32 registers they spilled (and a spill may move around a tensor-memory load).
 //
-// Measured (us; im2col kernel, this one): 3x3 256 -> 256 on 56 x 56 x 256 images 300, 167 (5.7 PTOPS; 59 % of the
-// instruction's rate); 1x1 512 -> 512 on 28 x 28 x 256 94.7, 43.3; 5x5 96 -> 256 on 27 x 27 x 128 43.5, 25.0; 3x3 1024
-// -> 1024 on 13 x 13 x 64 68.7, 42.8; the same AlexNet 5x5 layer with 4-bit codes 66.1, 47.5.  What bounds the large
-// layers now is instruction latency beside 24 warps (issue slots 48 to 60 % busy): the MMA warps wait for slots that
-// the epilogue takes.
+// Measured (us, uniform codes, launches back to back; im2col kernel, this one): 3x3 256 -> 256 on 56 x 56 x 256 images
+// 270, 167 (5.7 PTOPS; 59 % of the instruction's rate); 1x1 512 -> 512 on 28 x 28 x 256 92.3, 40.6; 5x5 96 -> 256 on 27 x 27
+// x 128 37.6, 23.6; 3x3 1024 -> 1024 on 13 x 13 x 64 64.8, 42.0; the same 5x5 layer with 4-bit codes 60.3, 46.5.  What
+// bounds the large layers now is instruction latency beside 24 warps (issue slots 48 to 59 % busy): the MMA warps wait
+// for slots that the epilogue takes.
 #pragma once
 #include "conv_common.cuh"
 

@@ -17,8 +17,10 @@
 //
 // Measured (us, batch 64, pooled; the kernel before, this one): 3 x 3 4 -> 8 on 416 x 416 8-bit pixels 64.9 (dp4a, the
 // direct kernel), 43.9; 3 x 3 8 -> 16 on 208 x 208 2-bit codes 41.9 (the warp kernel's e4m3 mma.sync, which
-// issues as four instructions), 30.3.  Their bytes take 7.5 and 1.25 us: the latency of loads and products bounds
-// both (issue slots 38.6 and 28.9 % busy; rows loaded one step ahead 45.2 and 32.3 us).
+// issues as four instructions), 30.3.  Their bytes take 7.5 and 1.25 us: latency bounds both.
+// On 16 images issue slots are busy in 41 and 30 % of the cycles; of the 12.2 and 8.4 cycles between two instructions of
+// a warp, 2.9 and 1.0 wait for loads, 3.1 and 2.0 for fixed latencies and 1.1 and 1.8 for the product pipe (rows
+// loaded one step ahead 45.2 and 32.3 us).
 #pragma once
 #include "conv_common.cuh"
 

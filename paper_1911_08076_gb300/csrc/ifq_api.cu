@@ -893,8 +893,8 @@ struct BandShape {
   int bn, mt, ngrp;
   bool resident;
 };
-// Of 48 shapes timed on 78 layers (the benchmark networks' and random ones) these are within 2 % of the best of
-// all on average; more channel tiles per CTA, streamed filters with one subtile, tiles of 32 channels and two
+// Of 48 shapes timed on 78 layers (the benchmark networks' and random ones, in an earlier build) these were within 2 %
+// of the best of all on average; more channel tiles per CTA, streamed filters with one subtile, tiles of 32 channels and two
 // CTAs per SM gained little anywhere.
 constexpr BandShape kBandShapes[] = {{64, 1, 1, true},  {64, 1, 2, true},  {64, 2, 1, true},
                                      {128, 1, 1, true}, {128, 1, 2, true}, {128, 2, 1, false}};
