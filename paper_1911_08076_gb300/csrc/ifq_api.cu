@@ -925,6 +925,14 @@ void band_fill(const ifq_conv_desc* d, const ConvGeom& g, const BandGeom& b, Ban
   a->div_HP = make_fastdiv((uint32_t)a->HP);
 }
 
+// What a grid of more than half of the SMs, or of about all, adds to a network: the CTAs of the next kernel (one an SM, too)
+// have fewer SMs to start on before it ends.  Timed alone, two shapes of one layer may take the same; in unfused Tiny-YOLO at
+// two images a layer of 86 instead of 152 CTAs takes 4 us less, in Tinier-YOLO at 16 one of 50 instead of 88 CTAs 4 us.
+// Chosen by the times of nine networks at 110 batches, 1.6 to 2 % below those with the estimates of single layers that
+// this replaces (1.4 % without this term, with single cases up to 11 % above); 900 to 2200 for the first step
+// differ by 0.1 %, and a cost that grows with the CTAs loses.
+double crowd_cycles(double ctas, int nsm) { return ctas > 0.9 * nsm ? 2300.0 : (2.0 * ctas > nsm ? 1500.0 : 0.0); }
+
 // Bytes of codes that an output pixel's share of a channel tile of bn stores one at a time, weighted with how many
 // cache lines a store instruction then touches: rows that are no multiple of `word` bytes are stored bytewise, else
 // the last channel tile's rest is.
@@ -1030,7 +1038,7 @@ bool band_try(const BandArgs& base, const BandShape& sh, int sbo, int nsm, BandP
   const double pace = std::max(std::max(mma, units * epi / 2), std::max(a.nchunk * chunk, stream));
   const double fits = wide ? std::ceil(cols * 4.0 / (32 * kBandEpi)) : 0.0;   // rounds of band_fit
   pl->cost = first + 5920.0 * fits + chunk + std::max(mma1, 0.94 * (a.nchunk - 1) * chunk) +
-             (ceil_div(a.mtiles, per) - 1) * pace;
+             (ceil_div(a.mtiles, per) - 1) * pace + crowd_cycles(pl->grid, nsm);
   return true;
 }
 
@@ -1044,7 +1052,7 @@ bool band_plan(const ifq_conv_desc* d, const ConvGeom& g, int nsm, double tc_cos
   if (!band_geom(d, g, &b)) return false;
   const int want = env_int("IFQ_BAND", 1);
   if (want == 0) return false;
-  if (want == 1 && 0.93 * tc_cost < 7500.0) return false;   // no estimate of band_try is below
+  if (want == 1 && 0.93 * tc_cost < 8570.0) return false;   // no estimate of band_try is below
   BandArgs base;
   band_fill(d, g, b, &base);
   base.y_codes = d->out_mode & IFQ_OUT_CODES ? (uint8_t*)16 : nullptr;   // (whether there is one)
@@ -1102,7 +1110,7 @@ double tc_cycles(const ifq_conv_desc* d, const ConvGeom& g, int nsm, int bn, int
   const double e1 = kEpi1[wide][j] * (acc ? 1.5 : 1.0) + bytes;
   const double e = kEpi[wide][j] * (acc ? (codes ? 1.685 : 1.56) : 1.0) + bytes;
   return 4320.0 + (ks == 2 ? 2850.0 : 0.0) + nk * kFirst[wide][i] + e1 +
-         (rounds - 1) * std::max(nk * kNext[wide][i] + 611.0, e);
+         (rounds - 1) * std::max(nk * kNext[wide][i] + 611.0, e) + crowd_cycles(tiles * ks, nsm);
 }
 
 // What the tensor-core path runs for a layer: the band kernel in a launch shape, or the im2col kernel with tiles of bn
